@@ -2,6 +2,7 @@
 // pair.  Included by one small translation unit per pair so the kernels compile in parallel.
 #pragma once
 
+#include "init.cuh"
 #include "launch.h"
 #include "step.cuh"
 #include "step_pair.cuh"
@@ -71,7 +72,12 @@ cudaError_t launch_init(const StepArgs<double>& a, int closure, const double* dr
                         const typename Store<ST>::R* ffield, typename Store<ST>::R* tau_field, cudaStream_t s) {
     dim3 g, b;
     lattice_grid(a.nx, a.ny, a.nzc, &g, &b);
-    k_init<L, ST><<<g, b, 0, s>>>(a, closure, drho, u, gu, ffield, tau_field);
+    const InitConst<InitX<ST>> k = init_const<L, InitX<ST>>(a, closure);
+    const InitConst<double> kd = init_const<L, double>(a, closure);
+    if (ffield || a.F[0] != 0.0 || a.F[1] != 0.0 || a.F[2] != 0.0)
+        k_init<L, ST, true><<<g, b, 0, s>>>(a, k, kd, drho, u, gu, ffield, tau_field);
+    else
+        k_init<L, ST, false><<<g, b, 0, s>>>(a, k, kd, drho, u, gu, ffield, tau_field);
     return cudaGetLastError();
 }
 

@@ -1,4 +1,4 @@
-// step.cuh -- the fused MRT lattice Boltzmann step and its read-out, init and sum kernels.
+// step.cuh -- the fused MRT lattice Boltzmann step and its read-out and sum kernels.
 //
 // A step pulls each node's 19 (or 9) pre-collision populations from the previous post-collision
 // buffer (f_i(x) = f*_i(x - c_i), Sec. 2 eq. (mrteq)), forms S by Yu's formula (eq. (LuoS)) or
@@ -1465,126 +1465,6 @@ __global__ void __launch_bounds__(128, step_min_blocks<L, ST>()) k_step(const St
     typename Store<ST>::R f[L::Q];
     pull<L, ST>(a, x, y, z, f);
     step_body<L, ST, CLOSURE, FORMULA, FORCE>(a, f, (z * a.ny + y) * a.nx + x);
-}
-
-// ------------------------------------------------------------------------------------------
-// initialisation from (drho, u, grad u), computed in double, un-streamed into the buffer
-
-template <class L, class ST>
-__global__ void __launch_bounds__(128) k_init(const StepArgs<double> a, int closure, const double* __restrict__ drho,
-                                              const double* __restrict__ u, const double* __restrict__ gu,
-                                              const typename Store<ST>::R* __restrict__ ffield,
-                                              typename Store<ST>::R* __restrict__ tau_field) {
-    using R = typename Store<ST>::R;
-    constexpr int Q = L::Q, D = L::D;
-    const int x = blockIdx.x * blockDim.x + threadIdx.x;
-    const int y = blockIdx.y * blockDim.y + threadIdx.y;
-    const int z = blockIdx.z + a.z0;
-    if (x >= a.nx || y >= a.ny) return;
-    const int nx = a.nx, ny = a.ny, nz = a.nz;
-    const long long N = (long long)nx * ny * nz;  // component offsets (up to 8N) exceed 2^31 on big grids
-    const int node = (z * ny + y) * nx + x;
-    const double r0 = a.rho0, ir0 = a.inv_rho0;
-    double j[3] = {0, 0, 0}, F[3] = {0, 0, 0};
-    for (int d = 0; d < D; ++d) j[d] = r0 * u[d * N + node];
-    for (int d = 0; d < D; ++d) F[d] = ffield ? double(ffield[d * N + node]) : a.F[d];
-    const double dr = drho[node];
-    // first-order viscous non-equilibrium moments of the given gradient (D3Q19: eq. (YuLuobasis);
-    // D2Q9 and D3Q15: the same first-order Chapman-Enskog moments worked out on their bases)
-    double mn[Q];
-#pragma unroll
-    for (int k = 0; k < Q; ++k) mn[k] = 0.0;
-    // the closure's tau at the prescribed gradient (explicit, since S is given); the lagged
-    // closure stores it as the tau of the first step
-    double G[3][3] = {{0, 0, 0}, {0, 0, 0}, {0, 0, 0}};
-    if (gu)
-        for (int p = 0; p < D; ++p)
-            for (int q = 0; q < D; ++q) G[p][q] = r0 * gu[(p * D + q) * N + node];
-    double tau_i = a.tau0;
-    if (closure != CL_NEWTON) {
-        double ss, tr = 0.0;
-        if (closure == CL_SMAG_DEV) tr = (G[0][0] + G[1][1] + G[2][2]) / D;  // traceless part only
-        const double e0 = G[0][0] - tr, e1 = G[1][1] - tr, e2 = D == 3 ? G[2][2] - tr : 0.0;
-        if (D == 3)
-            ss = e0 * e0 + e1 * e1 + e2 * e2 +
-                 0.5 * ((G[0][1] + G[1][0]) * (G[0][1] + G[1][0]) + (G[1][2] + G[2][1]) * (G[1][2] + G[2][1]) +
-                        (G[0][2] + G[2][0]) * (G[0][2] + G[2][0]));
-        else
-            ss = e0 * e0 + e1 * e1 + 0.5 * (G[0][1] + G[1][0]) * (G[0][1] + G[1][0]);
-        const double gnorm = sqrt(2.0 * ss) * ir0;
-        if (closure == CL_POWERLAW) {
-            tau_i = 0.5 + a.pl_k3 * pow(gnorm, a.pl_nm1);
-            if (!(tau_i >= a.pl_tau_min)) tau_i = a.pl_tau_min;
-            if (tau_i > a.pl_tau_max) tau_i = a.pl_tau_max;
-        } else {
-            tau_i = a.tau0 + a.smag_c3 * gnorm;
-        }
-    }
-    if (tau_field) tau_field[node] = R(tau_i);
-    if (gu) {
-        const double snu = closure == CL_NEWTON ? double(a.s[L::NU0]) : 1.0 / tau_i;
-        const double divj = G[0][0] + G[1][1] + G[2][2];
-        if constexpr (Q == 19) {
-            mn[1] = -38.0 / (3.0 * a.s[1]) * divj;
-            mn[9] = -2.0 / (3.0 * snu) * (3.0 * G[0][0] - divj);
-            mn[11] = -2.0 / (3.0 * snu) * (G[1][1] - G[2][2]);
-            mn[13] = -(G[1][0] + G[0][1]) / (3.0 * snu);
-            mn[14] = -(G[2][1] + G[1][2]) / (3.0 * snu);
-            mn[15] = -(G[0][2] + G[2][0]) / (3.0 * snu);
-        } else if constexpr (Q == 15) {
-            mn[1] = -2.0 / (3.0 * a.s[1]) * divj;
-            mn[9] = -2.0 / (3.0 * snu) * (3.0 * G[0][0] - divj);
-            mn[10] = -2.0 / (3.0 * snu) * (G[1][1] - G[2][2]);
-            mn[11] = -(G[1][0] + G[0][1]) / (3.0 * snu);
-            mn[12] = -(G[2][1] + G[1][2]) / (3.0 * snu);
-            mn[13] = -(G[0][2] + G[2][0]) / (3.0 * snu);
-        } else {
-            mn[1] = -2.0 * divj / a.s[1];
-            mn[7] = -2.0 * (G[0][0] - G[1][1]) / (3.0 * snu);
-            mn[8] = -(G[1][0] + G[0][1]) / (3.0 * snu);
-        }
-    }
-    double Dk[Q], add[Q];
-    sfor<Q>([&](auto k) { Dk[k] = mn[k] * (1.0 / norm2<L>(CV(k))); });
-    back_transform<L, (1u << Q) - 1u>(Dk, add);
-    const double jj = (j[0] * j[0] + j[1] * j[1] + j[2] * j[2]) * ir0;
-    const double jF = (j[0] * F[0] + j[1] * F[1] + j[2] * F[2]) * ir0;
-    ST* __restrict__ buf = static_cast<ST*>(a.dst);
-    const int dims[3] = {nx, ny, nz};
-    const int pos[3] = {x, y, z};
-    sfor<Q>([&](auto i) {
-        constexpr int cx = L::c(CV(i), 0), cy = L::c(CV(i), 1), cz = L::c(CV(i), 2);
-        const double w = double(L::wnum(CV(i))) / L::WDEN;
-        const double cj = cx * j[0] + cy * j[1] + cz * j[2];
-        const double cF = cx * F[0] + cy * F[1] + cz * F[2];
-        const double feq = w * (dr + 3.0 * cj + 4.5 * cj * cj * ir0 - 1.5 * jj);
-        const double fb = w * (3.0 * cF - 3.0 * jF + 9.0 * cj * cF * ir0);
-        double v = feq + add[i] - 0.5 * fb;
-        // un-stream: write where the pull of (node, i) will read
-        int s[3];
-        int nout = 0, face = -1;
-        for (int ax = 0; ax < 3; ++ax) {
-            const int cax = ax == 0 ? cx : (ax == 1 ? cy : cz);
-            s[ax] = pos[ax] - cax;
-            if (cax == 0 || (s[ax] >= 0 && s[ax] < dims[ax])) continue;
-            const int fc = 2 * ax + (s[ax] < 0 ? 0 : 1);
-            if ((a.wall_mask >> fc) & 1) {
-                ++nout;
-                face = fc;
-            } else {
-                s[ax] = s[ax] < 0 ? s[ax] + dims[ax] : s[ax] - dims[ax];
-            }
-        }
-        if (nout == 0) {
-            Store<ST>::st(buf + CV(i) * a.stride + (s[2] * ny + s[1]) * nx + s[0], R(v));
-        } else {
-            if (nout == 1 && ((a.lid_mask >> face) & 1)) {
-                const double cu = cx * a.lid[face][0] + cy * a.lid[face][1] + cz * a.lid[face][2];
-                v -= 6.0 * w * r0 * cu;
-            }
-            Store<ST>::st(buf + opp<L>(CV(i)) * a.stride + node, R(v));
-        }
-    });
 }
 
 // ------------------------------------------------------------------------------------------
