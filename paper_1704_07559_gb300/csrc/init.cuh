@@ -111,7 +111,7 @@ __device__ __forceinline__ void init_noneq(const InitConst<X>& k, X tau, const X
     X div = G[0][0] + G[1][1];
     if constexpr (L::D == 3) div = div + G[2][2];
     const X t3 = tau * XC<X>::c(-1.0 / 3.0);
-    X D[L::Q], O[L::NP];
+    X D[L::Q];
     sfor<L::Q>([&](auto i) { D[i] = X(0.0f); });
     auto shear = [&](int p, int q, int m) { return t3 * XC<X>::c(1.0 / m) * (G[p][q] + G[q][p]); };
     if constexpr (L::D == 3) {
@@ -125,17 +125,15 @@ __device__ __forceinline__ void init_noneq(const InitConst<X>& k, X tau, const X
         D[7] = t3 * XC<X>::c(2.0 / norm2<L>(7)) * (G[0][0] - G[1][1]);
         D[8] = shear(0, 1, norm2<L>(8));
     }
-    Xf<L>::template backward_eo<mask_viscous<L>()>(D, e0, e, O);
+    Xf<L>::viscous_even(D, e);
     const X m1 = k.e1 * div;
     e0 = X(float(L::T(1, 0))) * m1;  // the viscous rows of T have no rest entry
-    X by[3];                         // T_1a m1 by c_a.c_a = 1, 2, 3
     constexpr int ax = L::pa(0), dg = L::pa(L::NP - 1);
-    by[0] = X(float(L::T(1, ax))) * m1;
-    by[1] = X(float(L::T(1, dg))) * m1;
+    const X ma = X(float(L::T(1, ax))) * m1, md = X(float(L::T(1, dg))) * m1;  // axis, diagonal pairs
     sfor<L::NP>([&](auto p) {
         constexpr int i = L::pa(CV(p));
         constexpr bool axis = L::wnum(i) == L::wnum(ax);
-        e[p] = e[p] + by[axis ? 0 : 1];
+        e[p] = e[p] + (axis ? ma : md);
     });
 }
 

@@ -183,6 +183,16 @@ static_assert(basis_is_parity_split<D3Q19>(), "D3Q19 basis must split into even 
 static_assert(basis_is_parity_split<D2Q9>(), "D2Q9 basis must split into even and odd moments");
 static_assert(basis_is_parity_split<D3Q15>(), "D3Q15 basis must split into even and odd moments");
 
+// every viscous moment is even and has no rest entry
+template <class L>
+__host__ __device__ constexpr bool viscous_rows_even() {
+    for (int k = 0; k < L::Q; ++k)
+        if (L::viscous(k) && (!even_moment<L>(k) || L::T(k, 0) != 0)) return false;
+    return true;
+}
+static_assert(viscous_rows_even<D3Q19>() && viscous_rows_even<D2Q9>() && viscous_rows_even<D3Q15>(),
+              "viscous moments are even");
+
 // the rows of T are orthogonal (T^-1 = T^T diag(1/norm2) is used by every back-transform)
 template <class L>
 __host__ __device__ constexpr bool rows_orthogonal() {

@@ -145,11 +145,9 @@ __device__ __forceinline__ void step_pair(const StepArgs<float>& a, const F2 (&f
         });
     } else {
         // Chai route: the non-equilibrium distributions f - f_eq + Fbar/2 (opposite-pair form), their
-        // moments mn = T fn, Omega = T^-1 L mn back in distribution space (even parts: only those
-        // enter the contraction) and S = -N / (2 rho0 cs^2) with N = sum_i c_i c_i Omega_i.  The
-        // post-collision state is then formed from the same mn as f* = T^-1 m*, m*_k = m_eq_k +
-        // TF_k/2 + (1 - s_k) mn_k (the moments of f are mn + m_eq - TF/2), so neither f nor fn has to
-        // stay live across the transforms.
+        // moments mn = T fn, and S from them with the contraction folded into T^-1 (chai_contract).
+        // The post-collision state is formed from the same mn as f* = T^-1 m*, m*_k = m_eq_k + TF_k/2 +
+        // (1 - s_k) mn_k (the moments of f are mn + m_eq - TF/2), so neither f nor fn has to stay live.
         drho = f[0];
         sfor<NP>([&](auto p) { drho += P[p]; });
         sfor<L::D>([&](auto d) {
@@ -164,53 +162,42 @@ __device__ __forceinline__ void step_pair(const StepArgs<float>& a, const F2 (&f
             noneq_pairs<L, FORCE>(f[0], P, Dd, drho, j, u, F, fn0, Pn, Dn);
             Xf<L>::forward(fn0, Pn, Dn, mn);
         }
-        const R kS = R(-1.5f) * ir0;
-        if constexpr (CLOSURE == CL_NEWTON) {
-            snu = R(a.s[L::NU0]);  // with fixed rates S is a read-out only, not needed by the step
-        } else {
-            R Df[Q], Dv[Q];
-            sfor<Q>([&](auto k) {
-                constexpr double inv_n = 1.0 / norm2<L>(CV(k));
-                if constexpr (L::conserved(CV(k)) || L::viscous(CV(k)))
-                    Df[k] = R(0.0f);
-                else
-                    Df[k] = R(a.skn[k]) * mn[k];
-                if constexpr (L::viscous(CV(k)))
-                    Dv[k] = cst<R>(inv_n) * mn[k];
-                else
-                    Dv[k] = R(0.0f);
-            });
-            static_assert(viscous_moments_even<L>(), "viscous moments must be even");
-            R Ef0, Ef[NP], Of[NP], Ev0, Ev[NP], Ovd[NP];
-            Xf<L>::template backward_eo<mask_nonconserved<L>() & ~mask_viscous<L>()>(Df, Ef0, Ef, Of);
-            Xf<L>::template backward_eo<mask_viscous<L>()>(Dv, Ev0, Ev, Ovd);
-            R Nf[NS], Nv[NS], A[NS], B[NS];
-            contract_even<L>(Ef, Nf);
-            contract_even<L>(Ev, Nv);
-#pragma unroll
-            for (int c = 0; c < NS; ++c) {
-                A[c] = kS * Nf[c];
-                B[c] = kS * Nv[c];
-            }
-            solve_tau_pair<L, CLOSURE>(A, B, a, snu);
-        }
+        // G_k of the rate-independent moments before the closure, as on the Yu route
+        R Dn[Q];
         {
             R meq[Q], TF[Q];
             Eq<L>::meq(drho, j, u, meq);
             if constexpr (FORCE) Eq<L>::tforce(u, F, TF);
             sfor<Q>([&](auto k) {
                 constexpr double inv_n = 1.0 / norm2<L>(CV(k));
-                const bool has_tf = FORCE && !Eq<L>::ghost(CV(k)) && CV(k) != 0;
+                constexpr bool has_tf = FORCE && !Eq<L>::ghost(CV(k)) && CV(k) != 0;
+                if constexpr (L::viscous(CV(k))) {
+                    Dn[k] = cst<R>(inv_n) * mn[k];
+                } else if constexpr (!L::conserved(CV(k))) {
+                    Dn[k] = R(a.skn[k]) * mn[k];
+                }
                 // m_k + TF_k = mn_k + m_eq_k + TF_k / 2
-                R base = Eq<L>::ghost(CV(k)) ? mn[k] : mn[k] + meq[k];
+                R base = Eq<L>::ghost(CV(k)) ? mn[k] : (L::conserved(CV(k)) ? meq[k] : mn[k] + meq[k]);
                 if constexpr (has_tf) base = fma(R(0.5f), TF[k], base);
-                base = cst<R>(inv_n) * base;
-                if constexpr (L::conserved(CV(k)))
-                    G[k] = base;
-                else if constexpr (L::viscous(CV(k)))
-                    G[k] = fma(-(snu * cst<R>(inv_n)), mn[k], base);
+                if constexpr (L::conserved(CV(k)) || L::viscous(CV(k)))
+                    G[k] = cst<R>(inv_n) * base;
                 else
-                    G[k] = fma(R(-a.skn[k]), mn[k], base);
+                    G[k] = fma(cst<R>(inv_n), base, -Dn[k]);
+            });
+        }
+        if constexpr (CLOSURE == CL_NEWTON) {
+            // each viscous rate as given; with fixed rates S is a read-out only, not needed by the step
+            sfor<Q>([&](auto k) {
+                if constexpr (L::viscous(CV(k))) G[k] = fma(R(-a.s[k]), Dn[k], G[k]);
+            });
+        } else {
+            const R kS = R(-1.5f) * ir0;
+            R A[NS], B[NS];
+            chai_contract<L>(Dn, kS, [](int k) { return !L::conserved(k) && !L::viscous(k); }, A);
+            chai_contract<L>(Dn, kS, [](int k) { return L::viscous(k); }, B);
+            solve_tau_pair<L, CLOSURE>(A, B, a, snu);
+            sfor<Q>([&](auto k) {
+                if constexpr (L::viscous(CV(k))) G[k] = fma(-snu, Dn[k], G[k]);
             });
         }
     }
@@ -221,8 +208,8 @@ __device__ __forceinline__ void step_pair(const StepArgs<float>& a, const F2 (&f
 
 // Two x-adjacent nodes per thread (16-bit storage, nx even).  Bound to 7 resident blocks per SM
 // (72 registers) for both routes: measured on a GB300 against 8 blocks (Yu: channel -4%, 512^3 box
-// +1%) and, for the Chai route, 6 and 5 blocks (80 and 96 registers, fewer spilled values: channel
-// FP16 40.6 and 43.4 against 45.4 GLUPS, 512^3 box within 1%).
+// +1%; Chai: channel FP16 51.3 -> 48.9 GLUPS, D3Q15 BF16 59.5 -> 57.0, 256^3 box 62.9 -> 64.9) and, for
+// the Chai route, 6 and 5 blocks (channel 45.1 and 46.5, box 60.5).
 constexpr int PAIR_MIN_BLOCKS = 7;
 
 template <class L, class ST, int CLOSURE, int FORMULA, bool FORCE>
