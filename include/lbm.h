@@ -97,7 +97,9 @@ extern "C" {
 /* Model parameters (plain data, copied by lbm_create).  |S| = sqrt(2 S:S).  With a closure, S
  * and tau are solved together at each node by fixed-point sweeps on tau from the same
  * pre-collision state: Smagorinsky takes exactly smag_iters sweeps from tau0; the power law
- * sweeps from tau0 until |tau_new - tau| <= pl_tol * tau_new or pl_max_iter sweeps. */
+ * iterates until |F(tau) - tau| <= pl_tol * F(tau), F the closure's map, or pl_max_iter sweeps: plain
+ * sweeps from tau0, or, where those converge anyway (1/2 <= n <= 3/2, pl_max_iter >= 48, pl_tol <=
+ * 1e-5), Newton steps from a fitted guess to the same root. */
 typedef struct lbm_params {
     int precision;   /* LBM_FP64, LBM_FP32, LBM_FP16S, LBM_BF16S */
     int closure;     /* LBM_NEWTON, LBM_SMAG, LBM_POWERLAW, LBM_SMAG_LAGGED, LBM_SMAG_DEV */

@@ -13,6 +13,7 @@
 #include "adjoint.cuh"
 #include "adjoint_launch.h"
 #include "launch.h"
+#include "power_law.h"
 #include "step.cuh"
 
 struct lbm_ctx {
@@ -39,6 +40,7 @@ struct lbm_ctx {
     // several steps per launch: synchronisation words (error flag, ticket, per-unit step counts)
     // and the unit geometry; schedule is one of LBM_SCHEDULE_*
     int* sync;
+    lbm::PowerLawGuess pl_guess;  // power law: first guess of tau
     int stream_rows, stream_tiles;
     int schedule;
     long long n_steps, n_step_launches;  // steps advanced and step kernels launched by lbm_step
@@ -127,6 +129,7 @@ void fill_args(const lbm_ctx* c, lbm::StepArgs<R>* a) {
     a->pl_tau_min = R(c->p.pl_tau_min);
     a->pl_tau_max = R(c->p.pl_tau_max);
     a->pl_tol = R(c->p.pl_tol);
+    a->pl_guess = c->pl_guess;
     a->smag_iters = c->p.smag_iters;
     a->pl_max_iter = c->p.pl_max_iter;
     int wall = 0, lid = 0;
@@ -784,6 +787,9 @@ int lbm_create(lbm_ctx** out, int lattice, int nx, int ny, int nz, const double*
         for (int k = 0; k < 3; ++k)
             if (!is_finite(p.lid_u[f][k])) return bad("lid");
     if (p.force_field != 0 && p.force_field != 1) return bad("force_field");
+
+    if (p.closure == LBM_POWERLAW)
+        c->pl_guess = lbm::power_law_guess(p.pl_n, p.pl_k, p.pl_tau_min, p.pl_tau_max, p.pl_tol, p.pl_max_iter);
 
     // units of the multi-step launch: one z plane times enough rows for about 1024 nodes
     c->stream_rows = nx >= 1024 ? 1 : std::min(ny, 1024 / nx);

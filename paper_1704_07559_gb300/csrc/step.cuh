@@ -36,6 +36,7 @@
 #include <utility>
 
 #include "lattice.cuh"
+#include "power_law.h"
 
 
 namespace lbm {
@@ -156,17 +157,38 @@ struct Store<__nv_bfloat16> {
 
 __device__ __forceinline__ float r_abs(float x) { return fabsf(x); }
 __device__ __forceinline__ double r_abs(double x) { return fabs(x); }
-// Closure arithmetic: in FP32 the fast reciprocal / reciprocal-square-root / power intrinsics
-// (errors of a few ulp, far inside the FP32 tolerance of S); in FP64 the IEEE operations.
-__device__ __forceinline__ float c_rcp(float x) { return __fdividef(1.0f, x); }
+// Closure arithmetic: in FP32 the approximate reciprocal, reciprocal square root, logarithm and power of
+// two (errors of a few ulp, far inside the FP32 tolerance of S), in FP64 the IEEE operations.  The FP32
+// ones are the instructions that take subnormals as zero, without the scaling around them (channel
+// 256x128x128, 20 steps, Smagorinsky: FP16 Yu 61.1 -> 64.1 GLUPS, Chai 51.3 -> 53.8, FP32 Chai 41.7 -> 42.1):
+// tau lies above 1/2, and a squared strain below 2^-126 counts as zero.
+__device__ __forceinline__ float c_rcp(float x) {
+    float y;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
 __device__ __forceinline__ double c_rcp(double x) { return 1.0 / x; }
-__device__ __forceinline__ float c_sqrt(float x) { return x > 0.0f ? x * rsqrtf(x) : 0.0f; }
+__device__ __forceinline__ float c_sqrt(float x) {
+    float y;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return x >= 1.17549435e-38f ? x * y : 0.0f;
+}
 __device__ __forceinline__ double c_sqrt(double x) { return sqrt(x); }
+__device__ __forceinline__ float c_log2(float x) {
+    float y;
+    asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+__device__ __forceinline__ float c_exp2(float x) {
+    float y;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
 // |S|^(n-1) of the power-law closure from q2 = 2 S:S = |S|^2: in FP32 one fast power of q2 with
 // exponent (n-1)/2 (no square root; exactly 1 for n = 1; a q2 rounded below zero counts as zero,
 // as the square root's guard does), in FP64 the IEEE square root and power.
 __device__ __forceinline__ float strain_pow(float q2, float nm1) {
-    return nm1 == 0.0f ? 1.0f : __powf(fmaxf(q2, 0.0f), 0.5f * nm1);
+    return nm1 == 0.0f ? 1.0f : c_exp2(0.5f * nm1 * c_log2(fmaxf(q2, 0.0f)));
 }
 __device__ __forceinline__ double strain_pow(double q2, double nm1) { return pow(sqrt(q2), nm1); }
 
@@ -190,6 +212,7 @@ struct StepArgs {
     RS rho0, inv_rho0, tau0;
     RS smag_c3;            // 3 Cs^2
     RS pl_k3, pl_nm1, pl_tau_min, pl_tau_max, pl_tol;  // 3K, n-1, clamp, tolerance
+    PowerLawGuess pl_guess;  // first guess of tau
     int smag_iters, pl_max_iter;
     int wall_mask;         // bit f: face f is not periodic (wall or lid)
     int lid_mask;          // bit f: face f is a moving wall
@@ -806,10 +829,29 @@ __device__ __forceinline__ void affine(const R (&A)[L::NS], const R (&B)[L::NS],
     for (int c = 0; c < L::NS; ++c) S[c] = fma(s, B[c], A[c]);
 }
 
-// Fixed point for tau at one node from the quadratic |S|^2 = 2 (qa + qb2 s + qc s^2), s = 1/tau
-// (qa = A:A, qb2 = 2 A:B, qc = B:B: exact since S = A + s B).  Smagorinsky: `smag_iters` sweeps
-// from tau0, stopping early only when a sweep returns its input bit for bit (every later sweep
-// would too).  Power law: sweeps until |tau_new - tau| <= pl_tol tau_new or pl_max_iter sweeps.
+// First guess of the power law's tau (power_law.h): its root when the rate-free part of S vanishes.
+template <class RS>
+__device__ __forceinline__ RS power_law_start(RS qc, const StepArgs<RS>& a) {
+    const PowerLawGuess& g = a.pl_guess;
+    const float x = fmaf(g.ax, c_log2(2.0f * float(qc)), g.x0);
+    if (!(x > -1.0f)) return a.pl_tau_min;
+    if (x >= 1.0f) return a.pl_tau_max;
+    float v = g.p[POWER_LAW_DEGREE];
+    sfor<POWER_LAW_DEGREE>([&](auto i) { v = fmaf(v, x, g.p[POWER_LAW_DEGREE - 1 - CV(i)]); });
+    return RS(0.5f + c_exp2(v));
+}
+
+// tau at one node from the quadratic |S|^2 = 2 (qa + qb2 s + qc s^2), s = 1/tau (qa = A:A,
+// qb2 = 2 A:B, qc = B:B: exact since S = A + s B), as the fixed point of the closure's map F.
+// Smagorinsky: `smag_iters` sweeps from tau0, stopping early only when a sweep returns its input bit
+// for bit (every later sweep would too).  Power law: F(tau) = 1/2 + 3K |S|^(n-1), clamped, until
+// |F(tau) - tau| <= pl_tol F(tau) or pl_max_iter sweeps.  With a guess (the contractive range of n, see
+// power_law.h) the sweeps start from it and one that stays inside the clamps is followed by a Newton
+// step; there F has one fixed point, so the stopping rule accepts the same one.  A sweep costs 20
+// instructions and 3 special-function ones, a Newton step 8 and 1 more: from tau0 a node needs 8 to
+// 10 sweeps and a warp 12 to 18, from the guess 3 (4096^2 cavity, n = 0.5, developed flow, FP32
+// Yu / Chai 60.2 / 58.2 -> 83.0 / 78.7 GLUPS, 1024^2 FP64 0.37 -> 1.03; a cavity at rest, where two plain
+// sweeps did, 84.2 -> 83.3).
 template <int CLOSURE, class RS>
 __device__ __forceinline__ RS tau_fixed_point(RS qa, RS qb2, RS qc, const StepArgs<RS>& a) {
     RS tau = a.tau0;
@@ -821,14 +863,28 @@ __device__ __forceinline__ RS tau_fixed_point(RS qa, RS qb2, RS qc, const StepAr
             tau = tn;
         }
     } else {
+        const bool newton = a.pl_guess.on != 0;
+        if (newton) tau = power_law_start(qc, a);
         for (int it = 1; it <= a.pl_max_iter; ++it) {
             const RS s = c_rcp(tau);
-            RS tn = fma(a.pl_k3, strain_pow(RS(2) * fma(fma(qc, s, qb2), s, qa), a.pl_nm1), RS(0.5));
+            const RS r = fma(fma(qc, s, qb2), s, qa);
+            const RS t = fma(a.pl_k3, strain_pow(RS(2) * r, a.pl_nm1), RS(0.5));
+            RS tn = t;
             if (!(tn >= a.pl_tau_min)) tn = a.pl_tau_min;
             if (tn > a.pl_tau_max) tn = a.pl_tau_max;
-            const RS diff = r_abs(tn - tau);
+            const RS diff = tn - tau;
             tau = tn;
-            if (diff <= a.pl_tol * tn) break;
+            if (r_abs(diff) <= a.pl_tol * tn) break;
+            // Newton: dF/dtau = -e / r; not where it nears 1, and plain sweeps should eight steps not do
+            if (newton && tn == t && it <= 8) {
+                const RS e = (t - RS(0.5)) * a.pl_nm1 * (s * s) * fma(qc, s, RS(0.5) * qb2);
+                const RS den = r + e;
+                if (den > RS(0.25) * r) {
+                    tau = fma(-diff * e, c_rcp(den), tn);  // tau + diff r / (r + e), from F(tau)
+                    if (!(tau >= a.pl_tau_min)) tau = a.pl_tau_min;
+                    if (tau > a.pl_tau_max) tau = a.pl_tau_max;
+                }
+            }
         }
     }
     return tau;
@@ -1277,19 +1333,16 @@ readout:
 
 // One node per thread.  The bound names no minimum of resident blocks for the 3D lattices and
 // FP64: a minimum of one changes ptxas's register allocation (more registers, fewer resident
-// blocks).  FP32 D2Q9 is held to 16 blocks (32 registers, full occupancy), where the power-law
-// closure otherwise took 40-45 registers: with the one-power closure above, +4% on a 4096^2
-// power-law cavity (n = 0.5 and 1.5, both routes).  Chai's route with that closure spills at 32
-// registers and is held to 10 blocks: on a developed n = 0.5 cavity (many sweeps a node, bound by their
-// instructions) 56.6 / 56.6 / 58.5 / 59.0 GLUPS at 16 / 14 / 12 / 10 blocks.
-template <class L, class ST, int CLOSURE, int FORMULA>
+// blocks).  FP32 D2Q9 is held to 16 blocks (32 registers, full occupancy; the power law spills up to 12
+// values there): 4096^2 power-law cavity, developed n = 0.5 flow, Yu / Chai 83.0 / 78.7 GLUPS, at 12 blocks
+// 79.8 / 76.8, at 10 71.3 / 68.2.
+template <class L, class ST>
 constexpr int step_min_blocks() {
-    if (L::Q != 9 || sizeof(ST) != 4) return 0;
-    return CLOSURE == CL_POWERLAW && FORMULA == F_CHAI ? 10 : 16;
+    return (L::Q == 9 && sizeof(ST) == 4) ? 16 : 0;
 }
 
 template <class L, class ST, int CLOSURE, int FORMULA, bool FORCE>
-__global__ void __launch_bounds__(128, step_min_blocks<L, ST, CLOSURE, FORMULA>()) k_step(const StepArgs<typename Store<ST>::R> a) {
+__global__ void __launch_bounds__(128, step_min_blocks<L, ST>()) k_step(const StepArgs<typename Store<ST>::R> a) {
     pdl_wait();     // the previous step's stores are complete and visible from here on
     pdl_release();  // every block has started: the next step may be scheduled into freed slots
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
