@@ -1,4 +1,4 @@
-// instantiate.cuh -- defines the launch entry points of launch.h for one (lattice, storage)
+// instantiate.cuh -- defines the step and init entry points of launch.h for one (lattice, storage)
 // pair.  Included by one small translation unit per pair so the kernels compile in parallel.
 #pragma once
 
@@ -9,8 +9,8 @@
 
 namespace lbm {
 
-// Step kernel selection: one node per thread (k_step), except 16-bit storage with nx even and no
-// read-out, which runs two x-adjacent nodes per thread in packed FP32-pair arithmetic
+// Step kernel selection: one node per thread (k_step), except 16-bit storage with nx even,
+// which runs two x-adjacent nodes per thread in packed FP32-pair arithmetic
 // (k_step_pair_seq, step_pair.cuh: the 16-bit step is issue-bound, and the shared pull and the
 // pair instructions halve its arithmetic per node).  FP32 storage stays one node per thread: its
 // step already runs at the HBM bound, and it keeps the delta form, whose FP32 rounding acts on
@@ -18,14 +18,16 @@ namespace lbm {
 template <class L, class ST, int C, int F, bool FO>
 cudaError_t launch_form(const StepArgs<typename Store<ST>::R>& a, cudaStream_t s) {
     if constexpr (sizeof(ST) == 2) {
-        if (!a.readout && a.nx % 2 == 0) {
+        if (a.nx % 2 == 0) {
             dim3 g, b;
             lattice_grid(a.nx / 2, a.ny, a.nzc, &g, &b);
             return launch_pdl(k_step_pair_seq<L, ST, C, F, FO>, g, b, s, a);
         }
     }
+    // FP64 (bound by a pipe that each SM has its own share of): blocks of 64 spread a small lattice more
+    // evenly over the SMs (32^3: 512 blocks over 152 SMs instead of 256)
     dim3 g, b;
-    lattice_grid(a.nx, a.ny, a.nzc, &g, &b);
+    lattice_grid(a.nx, a.ny, a.nzc, &g, &b, sizeof(ST) == 8 ? 64 : 128);
     return launch_pdl(k_step<L, ST, C, F, FO>, g, b, s, a);
 }
 
@@ -81,15 +83,6 @@ cudaError_t launch_init(const StepArgs<double>& a, int closure, const double* dr
     return cudaGetLastError();
 }
 
-template <class L, class ST>
-cudaError_t launch_sums(const StepArgs<typename Store<ST>::R>& a, double* partial, double* out, cudaStream_t s) {
-    k_sums<L, ST><<<SUM_BLOCKS, SUM_THREADS, 0, s>>>(a, partial);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    k_sums_final<<<1, 256, 0, s>>>(partial, SUM_BLOCKS, 1 + L::D, out);
-    return cudaGetLastError();
-}
-
 }  // namespace lbm
 
 #define LBM_DEFINE_ENTRY(TAG, L, ST, EXTRA_CLOSURES)                                                         \
@@ -102,8 +95,5 @@ cudaError_t launch_sums(const StepArgs<typename Store<ST>::R>& a, double* partia
                            const double* gu, const Store<ST>::R* ffield, Store<ST>::R* tau_field,            \
                            cudaStream_t s) {                                                                 \
         return launch_init<L, ST>(a, closure, drho, u, gu, ffield, tau_field, s);                            \
-    }                                                                                                        \
-    cudaError_t sums_##TAG(const StepArgs<Store<ST>::R>& a, double* partial, double* out, cudaStream_t s) {  \
-        return launch_sums<L, ST>(a, partial, out, s);                                                       \
     }                                                                                                        \
     }

@@ -9,10 +9,11 @@ namespace lbm {
 template <class R>
 struct StepArgs;
 
-// geometry of a lattice launch: 128-thread blocks covering x (and several y rows when nx is small)
-inline void lattice_grid(int nx, int ny, int nz, dim3* grid, dim3* block) {
-    const int bx = nx <= 32 ? 32 : (nx <= 64 ? 64 : 128);
-    const int by = 128 / bx;
+// geometry of a lattice launch: blocks of `threads` (128) covering x (and several y rows when nx is small)
+inline void lattice_grid(int nx, int ny, int nz, dim3* grid, dim3* block, int threads = 128) {
+    int bx = nx <= 32 ? 32 : (nx <= 64 ? 64 : 128);
+    if (bx > threads) bx = threads;
+    const int by = threads / bx;
     *block = dim3(bx, by, 1);
     *grid = dim3((nx + bx - 1) / bx, (ny + by - 1) / by, nz);
 }
@@ -20,8 +21,8 @@ inline void lattice_grid(int nx, int ny, int nz, dim3* grid, dim3* block) {
 // Programmatic dependent launch of a step (or adjoint step) kernel: consecutive steps overlap launch and block
 // scheduling with the previous step's tail (the kernel waits for the previous one before its
 // first load).
-template <class K, class A>
-cudaError_t launch_pdl(K kernel, dim3 g, dim3 b, cudaStream_t s, const A& a) {
+template <class K, class... A>
+cudaError_t launch_pdl(K kernel, dim3 g, dim3 b, cudaStream_t s, const A&... a) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = g;
     cfg.blockDim = b;
@@ -32,7 +33,7 @@ cudaError_t launch_pdl(K kernel, dim3 g, dim3 b, cudaStream_t s, const A& a) {
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kernel, a);
+    return cudaLaunchKernelEx(&cfg, kernel, a...);
 }
 
 // Several steps in one launch (step_stream.cuh): the library-owned synchronisation words and the
@@ -47,6 +48,16 @@ struct StreamCtl {
     int first_step;  // 0; 1 only for the diagnostic that makes every dependency wait run out
     long long ring;  // 0: two buffers; else step k's buffers are the first ones shifted by k * ring elements
 };
+
+// floor(n / d) for 0 <= n < 2^31 as (n m) >> s
+struct FastDiv {
+    unsigned m, s;
+};
+inline FastDiv fast_div(unsigned d) {
+    unsigned l = 0;
+    while ((1ull << l) < d) ++l;
+    return {(unsigned)(((1ull << (31 + l)) + d - 1) / d), 31 + l};
+}
 
 constexpr int SUM_BLOCKS = 608;  // 4 blocks per SM on 152 SMs; partial rows in scratch
 
@@ -72,7 +83,10 @@ cudaError_t halo_copy(const HaloArgs& h, int pack, int elem_bytes, cudaStream_t 
     cudaError_t step_##TAG(const StepArgs<R>& a, int closure, int formula, int force, cudaStream_t s);   \
     cudaError_t init_##TAG(const StepArgs<double>& a, int closure, const double* drho, const double* u, \
                            const double* gu, const R* ffield, R* tau_field, cudaStream_t s);             \
-    cudaError_t sums_##TAG(const StepArgs<R>& a, double* partial, double* out, cudaStream_t s);
+    cudaError_t strain_##TAG(const StepArgs<R>& a, int closure, int formula, int force, cudaStream_t s);  \
+    cudaError_t macro_##TAG(const StepArgs<R>& a, int formula, int force, cudaStream_t s);                \
+    cudaError_t sums_##TAG(const StepArgs<R>& a, double* partial, int blocks, const int* flag, double* out, \
+                           cudaStream_t s);
 
 #define LBM_DECLARE_STREAM_ENTRY(TAG, R)                                                                      \
     cudaError_t stream_##TAG(const StepArgs<R>& a0, const StepArgs<R>& a1, const StreamCtl& c, int closure, \

@@ -41,15 +41,6 @@ cudaError_t scratch_for_current_device(double** out) {
     return cudaSuccess;
 }
 
-template <class L, class ST>
-cudaError_t run(const lbm::StepArgs<typename lbm::Store<ST>::R>& a, int blocks, double* scratch, cudaStream_t s) {
-    lbm::k_sums<L, ST><<<blocks, lbm::SUM_THREADS, 0, s>>>(a, scratch);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    lbm::k_sums_final<<<1, 256, 0, s>>>(scratch, blocks, 1 + L::D, scratch + MAX_BLOCKS * WIDTH);
-    return cudaGetLastError();
-}
-
 template <class R>
 void fill(lbm::StepArgs<R>* a, int q, int nx, int ny, int nz, const lbm_params* p, const double* force,
           const void* f, int64_t stride, int elem, const void* ffield) {
@@ -116,30 +107,31 @@ extern "C" int lbm_sums_noalloc(int lattice, int nx, int ny, int nz, const lbm_p
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     cudaError_t e;
     const int nb = (int)blocks;
+    double* result = scratch + MAX_BLOCKS * WIDTH;
     if (p->precision == LBM_FP64) {
         lbm::StepArgs<double> a;
         fill(&a, lattice, nx, ny, nz, p, force, f, stride, elem, force_field);
-        e = lattice == LBM_D3Q19   ? run<lbm::D3Q19, double>(a, nb, scratch, s)
-            : lattice == LBM_D3Q15 ? run<lbm::D3Q15, double>(a, nb, scratch, s)
-                                   : run<lbm::D2Q9, double>(a, nb, scratch, s);
+        e = lattice == LBM_D3Q19   ? lbm::sums_d3q19_f64(a, scratch, nb, nullptr, result, s)
+            : lattice == LBM_D3Q15 ? lbm::sums_d3q15_f64(a, scratch, nb, nullptr, result, s)
+                                   : lbm::sums_d2q9_f64(a, scratch, nb, nullptr, result, s);
     } else {
         lbm::StepArgs<float> a;
         fill(&a, lattice, nx, ny, nz, p, force, f, stride, elem, force_field);
         if (lattice == LBM_D2Q9)
-            e = run<lbm::D2Q9, float>(a, nb, scratch, s);
+            e = lbm::sums_d2q9_f32(a, scratch, nb, nullptr, result, s);
         else if (lattice == LBM_D3Q15)
-            e = p->precision == LBM_FP32    ? run<lbm::D3Q15, float>(a, nb, scratch, s)
-                : p->precision == LBM_FP16S ? run<lbm::D3Q15, __half>(a, nb, scratch, s)
-                                            : run<lbm::D3Q15, __nv_bfloat16>(a, nb, scratch, s);
+            e = p->precision == LBM_FP32    ? lbm::sums_d3q15_f32(a, scratch, nb, nullptr, result, s)
+                : p->precision == LBM_FP16S ? lbm::sums_d3q15_f16(a, scratch, nb, nullptr, result, s)
+                                            : lbm::sums_d3q15_bf16(a, scratch, nb, nullptr, result, s);
         else if (p->precision == LBM_FP32)
-            e = run<lbm::D3Q19, float>(a, nb, scratch, s);
+            e = lbm::sums_d3q19_f32(a, scratch, nb, nullptr, result, s);
         else if (p->precision == LBM_FP16S)
-            e = run<lbm::D3Q19, __half>(a, nb, scratch, s);
+            e = lbm::sums_d3q19_f16(a, scratch, nb, nullptr, result, s);
         else
-            e = run<lbm::D3Q19, __nv_bfloat16>(a, nb, scratch, s);
+            e = lbm::sums_d3q19_bf16(a, scratch, nb, nullptr, result, s);
     }
     if (e != cudaSuccess) return LBM_ERR_CUDA;
-    e = cudaMemcpyAsync(out, scratch + MAX_BLOCKS * WIDTH, sizeof(double) * (1 + d), cudaMemcpyDeviceToHost, s);
+    e = cudaMemcpyAsync(out, result, sizeof(double) * (1 + d), cudaMemcpyDeviceToHost, s);
     if (e != cudaSuccess) return LBM_ERR_CUDA;
     e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) return LBM_ERR_CUDA;

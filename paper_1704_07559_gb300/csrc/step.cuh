@@ -1,4 +1,4 @@
-// step.cuh -- the fused MRT lattice Boltzmann step and its read-out and sum kernels.
+// step.cuh -- the fused MRT lattice Boltzmann step.
 //
 // A step pulls each node's 19 (or 9) pre-collision populations from the previous post-collision
 // buffer (f_i(x) = f*_i(x - c_i), Sec. 2 eq. (mrteq)), forms S by Yu's formula (eq. (LuoS)) or
@@ -199,7 +199,6 @@ template <class RS>
 struct StepArgs {
     int nx, ny, nz;
     int z0, nzc;           // planes computed: [z0, z0 + nzc) (all, or the owned planes between halo planes)
-    int readout;           // 0: step (write f*); 1: write S/tau/drho/u of the pre-collision state
     long long stride;      // elements between population arrays
     const void* src;       // post-collision buffer of the previous step
     void* dst;             // post-collision buffer of this step
@@ -973,7 +972,7 @@ __device__ __forceinline__ RS tau_deviatoric(RS qc, const StepArgs<RS>& a) {
 // Returns tau, sets snu = 1/tau and S = A + snu B.  The lagged closure collides with tau_prev, the
 // tau stored at `node` (loaded by the caller together with the populations), and in a step (not a
 // read-out) stores tau0 + 3 Cs^2 |S| there for the next step.
-template <class L, class R, int CLOSURE, class RS>
+template <class L, class R, int CLOSURE, bool STEP, class RS>
 __device__ __forceinline__ R solve_tau(const R (&A)[L::NS], const R (&B)[L::NS], const StepArgs<RS>& a,
                                        R (&S)[L::NS], R& snu, int node, R tau_prev = R(0.0f)) {
     if constexpr (CLOSURE == CL_NEWTON) {
@@ -984,7 +983,8 @@ __device__ __forceinline__ R solve_tau(const R (&A)[L::NS], const R (&B)[L::NS],
         const R tau = tau_prev;
         snu = c_rcp(tau);
         affine<L>(A, B, snu, S);
-        if (!a.readout) st_keep(a.tau_field + node, RS(fma(a.smag_c3, c_sqrt(RS(2) * strain_dot<L>(S, S)), a.tau0)));
+        if constexpr (STEP)
+            st_keep(a.tau_field + node, RS(fma(a.smag_c3, c_sqrt(RS(2) * strain_dot<L>(S, S)), a.tau0)));
         return tau;
     } else if constexpr (CLOSURE == CL_SMAG_DEV) {
         const R tau = tau_deviatoric(strain_dot<L>(B, B), a);
@@ -1184,110 +1184,97 @@ __device__ __forceinline__ void pull2(const StepArgs<float>& a, int x0, int y, i
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
-// Everything of a step after the pull, for the node(s) starting at `node`: moments, strain rate
-// by the chosen route, closure, relaxation, force, and either the store of f* or (readout) the
-// store of S, tau, drho and u.  ds shifts the populations' destination by that many elements (a
-// launch that writes each step to its own buffer of a ring); the pull's es does the same for the
-// source.
-template <class L, class ST, int CLOSURE, int FORMULA, bool FORCE>
-__device__ __forceinline__ void step_body(const StepArgs<typename Store<ST>::R>& a, typename Store<ST>::R (&f)[L::Q],
-                                          int node, long long ds = 0) {
-    using RS = typename Store<ST>::R;
-    using R = RS;
-    constexpr int Q = L::Q, NS = L::NS, NP = L::NP;
-    const long long N = (long long)a.nx * a.ny * a.nz;  // component offsets c*N exceed 2^31 on big grids
-
-    R P[NP], Dd[NP];
-    sfor<NP>([&](auto p) {
+// opposite-pair sums and differences of the pulled populations
+template <class L, class R>
+__device__ __forceinline__ void pair_sums(const R (&f)[L::Q], R (&P)[L::NP], R (&Dd)[L::NP]) {
+    sfor<L::NP>([&](auto p) {
         P[p] = f[L::pa(CV(p))] + f[L::pb(CV(p))];
         Dd[p] = f[L::pa(CV(p))] - f[L::pb(CV(p))];
     });
-    R F[3] = {R(0.0f), R(0.0f), R(0.0f)};
+}
+
+// the node's force density: its entry of the force field, or the uniform force
+template <class L, bool FORCE, class RS, class R>
+__device__ __forceinline__ void node_force(const StepArgs<RS>& a, int node, R (&F)[3]) {
+    sfor<3>([&](auto d) { F[d] = R(0.0f); });
     if constexpr (FORCE) {
         if (a.force_field) {
+            const long long N = (long long)a.nx * a.ny * a.nz;  // component offsets exceed 2^31 on big grids
             sfor<L::D>([&](auto d) { F[d] = ld_keep(a.force_field + CV(d) * N + node); });
         } else {
             sfor<L::D>([&](auto d) { F[d] = R(a.F[d]); });
         }
     }
-    // the lagged closure's stored tau, loaded next to the populations so its latency overlaps theirs
-    // (an asm volatile load keeps it there instead of next to its use after the moment arithmetic)
-    R tau_prev = R(0.0f);
-    if constexpr (CLOSURE == CL_SMAG_LAGGED) tau_prev = load_early_keep(a.tau_field + node);
-    const R ir0 = R(a.inv_rho0);
-    R drho, j[3] = {R(0.0f), R(0.0f), R(0.0f)}, u[3] = {R(0.0f), R(0.0f), R(0.0f)};
-    R S[NS], tau, snu;
-    R out[Q];  // f*_i = f_i - out_i
+}
 
-    // non-equilibrium moments mn = T (f - f_eq + Fbar/2) of the non-conserved rows
-    R mn[Q];
+// delta rho, j = sum c f + F/2 and u = j / rho0; on the Yu route with all moments m = T f
+template <class L, int FORMULA, bool FORCE, class R>
+__device__ __forceinline__ void conserved_moments(R f0, const R (&P)[L::NP], const R (&Dd)[L::NP], const R (&F)[3],
+                                                  R ir0, R& drho, R (&j)[3], R (&u)[3], R (&m)[L::Q]) {
+    j[2] = u[2] = R(0.0f);
     if constexpr (FORMULA == F_YU) {
-        // Yu route: the moments of f less the closed-form equilibrium moments
-        R m[Q], meq[Q];
-        Xf<L>::forward(f[0], P, Dd, m);
+        Xf<L>::forward(f0, P, Dd, m);
         drho = m[0];
         j[0] = FORCE ? fma(R(0.5f), F[0], m[3]) : m[3];
         j[1] = FORCE ? fma(R(0.5f), F[1], m[5]) : m[5];
         if constexpr (L::D == 3) j[2] = FORCE ? fma(R(0.5f), F[2], m[7]) : m[7];
-        sfor<L::D>([&](auto d) { u[d] = j[d] * ir0; });
+    } else {
+        drho = f0;
+        sfor<L::NP>([&](auto p) { drho += P[p]; });
+        sfor<L::D>([&](auto d) {
+            R acc = nzero<R>();
+            sfor<L::NP>([&](auto p) { acc = cadd<L::c(L::pa(CV(p)), CV(d))>(acc, Dd[p]); });
+            j[d] = FORCE ? fma(R(0.5f), F[d], acc) : acc;
+        });
+    }
+    sfor<L::D>([&](auto d) { u[d] = j[d] * ir0; });
+}
+
+// non-equilibrium moments mn = T (f - f_eq + Fbar/2) of the non-conserved rows, with TF = T Fbar.  Yu
+// route: the moments of f less the closed-form equilibrium moments.  Chai route: the moments of the
+// non-equilibrium distributions (in opposite-pair form).
+template <class L, int FORMULA, bool FORCE, class R>
+__device__ __forceinline__ void noneq_moments(R f0, const R (&P)[L::NP], const R (&Dd)[L::NP], const R (&F)[3],
+                                              R drho, const R (&j)[3], const R (&u)[3], const R (&m)[L::Q],
+                                              R (&mn)[L::Q], R (&TF)[L::Q]) {
+    if constexpr (FORCE) Eq<L>::tforce(u, F, TF);
+    if constexpr (FORMULA == F_YU) {
+        R meq[L::Q];
         Eq<L>::meq(drho, j, u, meq);
-        sfor<Q>([&](auto k) {
+        sfor<L::Q>([&](auto k) {
             if constexpr (L::conserved(CV(k)))
                 mn[k] = R(0.0f);
             else if constexpr (Eq<L>::ghost(CV(k)))
                 mn[k] = m[k];
+            else if constexpr (FORCE)
+                mn[k] = fma(R(0.5f), TF[k], m[k] - meq[k]);
             else
                 mn[k] = m[k] - meq[k];
         });
     } else {
-        // Chai route: the moments of the non-equilibrium distributions (in opposite-pair form)
-        drho = f[0];
-        sfor<NP>([&](auto p) { drho += P[p]; });
-        sfor<L::D>([&](auto d) {
-            R acc = nzero<R>();
-            sfor<NP>([&](auto p) { acc = cadd<L::c(L::pa(CV(p)), CV(d))>(acc, Dd[p]); });
-            j[d] = FORCE ? fma(R(0.5f), F[d], acc) : acc;
-            u[d] = j[d] * ir0;
-        });
-        R fn0, Pn[NP], Dn[NP];
-        noneq_pairs<L, FORCE>(f[0], P, Dd, drho, j, u, F, fn0, Pn, Dn);
+        R fn0, Pn[L::NP], Dn[L::NP];
+        noneq_pairs<L, FORCE>(f0, P, Dd, drho, j, u, F, fn0, Pn, Dn);
         Xf<L>::forward(fn0, Pn, Dn, mn);
     }
-    // every collision increment D_k = (s_k mn_k - TF_k) / |T_k|^2 that does not involve an unknown
-    // viscous rate is finished before the closure, so only the viscous moments (and their force terms)
-    // stay live across the fixed point.  Chai's formula takes each viscous rate as given.
-    constexpr bool KNOWN = CLOSURE == CL_NEWTON && FORMULA == F_CHAI;
-    R Dk[Q], tv[Q], A[NS], B[NS];
-    {
-        R TF[Q];
-        if constexpr (FORCE) Eq<L>::tforce(u, F, TF);
-        sfor<Q>([&](auto k) {
-            constexpr double inv_n = 1.0 / norm2<L>(CV(k));
-            constexpr bool has_tf = FORCE && !Eq<L>::ghost(CV(k));
-            if constexpr (L::conserved(CV(k))) {
-                if constexpr (FORCE)
-                    Dk[k] = cst<R>(-inv_n) * TF[k];
-                else
-                    Dk[k] = R(0.0f);
-            } else {
-                if constexpr (FORMULA == F_YU && has_tf) mn[k] = fma(R(0.5f), TF[k], mn[k]);
-                if constexpr (has_tf) tv[k] = cst<R>(-inv_n) * TF[k];
-                if constexpr (!L::viscous(CV(k)) || KNOWN) {
-                    if constexpr (has_tf)
-                        Dk[k] = fma(R(a.skn[k]), mn[k], tv[k]);
-                    else
-                        Dk[k] = R(a.skn[k]) * mn[k];
-                }
-            }
-        });
-    }
+}
+
+// Chai's formula with fixed rates takes each viscous rate as given, so S does not split
+template <int CLOSURE, int FORMULA>
+constexpr bool rates_known() {
+    return CLOSURE == CL_NEWTON && FORMULA == F_CHAI;
+}
+
+// S = A + s_nu B by the route's formula (B = 0 with the rates known)
+template <class L, int CLOSURE, int FORMULA, class RS, class R>
+__device__ __forceinline__ void strain_split(const StepArgs<RS>& a, const R (&mn)[L::Q], R ir0, R (&A)[L::NS],
+                                             R (&B)[L::NS]) {
     if constexpr (FORMULA == F_YU) {
         Eq<L>::yu_split(mn, R(a.s[1] * RS(Eq<L>::YU_A)) * ir0, ir0, A, B);
     } else {
-        // S = A + s_nu B: the viscous part per unit rate, or with the given rates (then B = 0)
-        const R kS = R(-1.5f) * ir0;
-        R Dn[Q];
-        sfor<Q>([&](auto k) {
+        constexpr bool KNOWN = rates_known<CLOSURE, FORMULA>();
+        const R kS = R(-1.5f) * ir0;  // -1 / (2 rho0 cs^2)
+        R Dn[L::Q];
+        sfor<L::Q>([&](auto k) {
             if constexpr (L::viscous(CV(k)) && !KNOWN)
                 Dn[k] = cst<R>(1.0 / norm2<L>(CV(k))) * mn[k];
             else if constexpr (!L::conserved(CV(k)))
@@ -1295,13 +1282,60 @@ __device__ __forceinline__ void step_body(const StepArgs<typename Store<ST>::R>&
         });
         chai_contract<L>(Dn, kS, [](int k) { return !L::conserved(k) && (KNOWN || !L::viscous(k)); }, A);
         if constexpr (KNOWN)
-            sfor<NS>([&](auto c) { B[c] = R(0.0f); });
+            sfor<L::NS>([&](auto c) { B[c] = R(0.0f); });
         else
             chai_contract<L>(Dn, kS, [](int k) { return L::viscous(k); }, B);
     }
-    tau = solve_tau<L, R, CLOSURE>(A, B, a, S, snu, node, tau_prev);
-    if (a.readout) goto readout;
+}
+
+// Everything of a step after the pull, for the node `node`: moments, strain rate by the chosen route,
+// closure, relaxation, force, and the store of f*.  ds shifts the populations' destination by that many
+// elements (a launch that writes each step to its own buffer of a ring); the pull's es does the same for
+// the source.
+template <class L, class ST, int CLOSURE, int FORMULA, bool FORCE>
+__device__ __forceinline__ void step_body(const StepArgs<typename Store<ST>::R>& a, typename Store<ST>::R (&f)[L::Q],
+                                          int node, long long ds = 0) {
+    using R = typename Store<ST>::R;
+    constexpr int Q = L::Q, NS = L::NS, NP = L::NP;
+
+    R P[NP], Dd[NP], F[3];
+    pair_sums<L>(f, P, Dd);
+    node_force<L, FORCE>(a, node, F);
+    // the lagged closure's stored tau, loaded next to the populations so its latency overlaps theirs
+    // (an asm volatile load keeps it there instead of next to its use after the moment arithmetic)
+    R tau_prev = R(0.0f);
+    if constexpr (CLOSURE == CL_SMAG_LAGGED) tau_prev = load_early_keep(a.tau_field + node);
+    const R ir0 = R(a.inv_rho0);
+    R drho, j[3], u[3], m[Q], mn[Q], TF[Q];
+    conserved_moments<L, FORMULA, FORCE>(f[0], P, Dd, F, ir0, drho, j, u, m);
+    noneq_moments<L, FORMULA, FORCE>(f[0], P, Dd, F, drho, j, u, m, mn, TF);
+    // every collision increment D_k = (s_k mn_k - TF_k) / |T_k|^2 that does not involve an unknown
+    // viscous rate is finished before the closure, so only the viscous moments (and their force terms)
+    // stay live across the fixed point
+    constexpr bool KNOWN = rates_known<CLOSURE, FORMULA>();
+    R Dk[Q], tv[Q];
+    sfor<Q>([&](auto k) {
+        constexpr double inv_n = 1.0 / norm2<L>(CV(k));
+        constexpr bool has_tf = FORCE && !Eq<L>::ghost(CV(k));
+        if constexpr (L::conserved(CV(k))) {
+            if constexpr (FORCE)
+                Dk[k] = cst<R>(-inv_n) * TF[k];
+            else
+                Dk[k] = R(0.0f);
+        } else {
+            if constexpr (has_tf) tv[k] = cst<R>(-inv_n) * TF[k];
+            if constexpr (!L::viscous(CV(k)) || KNOWN) {
+                if constexpr (has_tf)
+                    Dk[k] = fma(R(a.skn[k]), mn[k], tv[k]);
+                else
+                    Dk[k] = R(a.skn[k]) * mn[k];
+            }
+        }
+    });
     if constexpr (!KNOWN) {
+        R A[NS], B[NS], S[NS], snu;
+        strain_split<L, CLOSURE, FORMULA>(a, mn, ir0, A, B);
+        solve_tau<L, R, CLOSURE, true>(A, B, a, S, snu, node, tau_prev);
         sfor<Q>([&](auto k) {
             if constexpr (L::viscous(CV(k))) {
                 constexpr double inv_n = 1.0 / norm2<L>(CV(k));
@@ -1312,23 +1346,10 @@ __device__ __forceinline__ void step_body(const StepArgs<typename Store<ST>::R>&
             }
         });
     }
-    // with a force, the conserved moments 3, 5, 7 (D2Q9: 3, 5) carry -TF_k; TF_0 = 0
+    // f*_i = f_i - out_i; with a force, the conserved moments 3, 5, 7 (D2Q9: 3, 5) carry -TF_k; TF_0 = 0
+    R out[Q];
     Xf<L>::template backward<FORCE ? mask_all_but_density<L>() : mask_nonconserved<L>()>(Dk, out);
-
     sfor<Q>([&](auto i) { Store<ST>::st(static_cast<ST*>(a.dstp[CV(i)]) + ds + node, f[i] - out[i]); });
-    return;
-
-readout:
-    if (a.S_out) {
-#pragma unroll
-        for (int c = 0; c < NS; ++c) a.S_out[c * N + node] = S[c];
-    }
-    if (a.tau_out) a.tau_out[node] = tau;
-    if (a.drho_out) a.drho_out[node] = drho;
-    if (a.u_out) {
-#pragma unroll
-        for (int d = 0; d < L::D; ++d) a.u_out[d * N + node] = u[d];
-    }
 }
 
 // One node per thread.  The bound names no minimum of resident blocks for the 3D lattices and
@@ -1353,76 +1374,5 @@ __global__ void __launch_bounds__(128, step_min_blocks<L, ST>()) k_step(const St
     pull<L, ST>(a, x, y, z, f);
     step_body<L, ST, CLOSURE, FORMULA, FORCE>(a, f, (z * a.ny + y) * a.nx + x);
 }
-
-// ------------------------------------------------------------------------------------------
-// global sums: each block walks whole rows (fixed assignment, so the result is reproducible);
-// each node's totals are formed in the compute type, then FP32 states accumulate them across nodes
-// with an error-free two-sum (hi, lo) pair per component, FP64 states in plain FP64; per-block
-// partials go to scratch as FP64 and one ordered pass adds them.
-
-constexpr int SUM_THREADS = 256;
-
-template <class R>
-struct Comp {
-    R hi = R(0), lo = R(0);
-    __device__ __forceinline__ void add(R x) {
-        if constexpr (sizeof(R) == 4) {
-            const R t = hi + x;
-            const R bp = t - hi;
-            lo += (hi - (t - bp)) + (x - bp);
-            hi = t;
-        } else {
-            hi += x;
-        }
-    }
-    __device__ __forceinline__ double value() const { return double(hi) + double(lo); }
-};
-
-template <class L, class ST>
-__global__ void __launch_bounds__(SUM_THREADS) k_sums(const StepArgs<typename Store<ST>::R> a, double* __restrict__ partial) {
-    using R = typename Store<ST>::R;
-    constexpr int D = L::D;
-    const long long N = (long long)a.nx * a.ny * a.nz;  // component offsets c*N exceed 2^31 on big grids
-    const int rows = a.ny * a.nzc;  // the computed planes only (a halo plane belongs to a neighbour)
-    Comp<R> acc[1 + D];
-    for (int r = blockIdx.x; r < rows; r += gridDim.x) {
-        const int y = r % a.ny, z = r / a.ny + a.z0;
-        for (int x = threadIdx.x; x < a.nx; x += blockDim.x) {
-            R f[L::Q];
-            pull<L, ST>(a, x, y, z, f);
-            // the node's own totals in plain arithmetic (19 values of one node), then one
-            // compensated add per component across nodes
-            R m0 = nzero<R>(), mj[3] = {nzero<R>(), nzero<R>(), nzero<R>()};
-            sfor<L::Q>([&](auto i) {
-                m0 += f[i];
-                sfor<D>([&](auto d) { mj[d] = cadd<L::c(CV(i), CV(d))>(mj[d], f[i]); });
-            });
-            const int n = (z * a.ny + y) * a.nx + x;
-            acc[0].add(m0);
-#pragma unroll
-            for (int d = 0; d < D; ++d)
-                acc[1 + d].add(fma(R(0.5), a.force_field ? a.force_field[d * N + n] : a.F[d], mj[d]));
-        }
-    }
-    __shared__ double red[SUM_THREADS / 32][1 + D];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-    for (int c = 0; c <= D; ++c) {
-        double v = acc[c].value();
-        for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-        if (lane == 0) red[warp][c] = v;
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        for (int c = 0; c <= D; ++c) {
-            double v = 0.0;
-            for (int w = 0; w < SUM_THREADS / 32; ++w) v += red[w][c];
-            partial[blockIdx.x * (1 + D) + c] = v;
-        }
-    }
-}
-
-// sums nblocks partial rows of width `width` in block order into out[width]
-__global__ void k_sums_final(const double* __restrict__ partial, int nblocks, int width, double* __restrict__ out);
 
 }  // namespace lbm
