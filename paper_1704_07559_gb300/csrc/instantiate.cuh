@@ -17,18 +17,18 @@ namespace lbm {
 // the collision increment only; FP64 is bound by its arithmetic.
 template <class L, class ST, int C, int F, bool FO>
 cudaError_t launch_form(const StepArgs<typename Store<ST>::R>& a, cudaStream_t s) {
+    dim3 g;
     if constexpr (sizeof(ST) == 2) {
         if (a.nx % 2 == 0) {
-            dim3 g, b;
-            lattice_grid(a.nx / 2, a.ny, a.nzc, &g, &b);
-            return launch_pdl(k_step_pair_seq<L, ST, C, F, FO>, g, b, s, a);
+            const NodeMap m = node_grid<2>(a, 128, &g);
+            return launch_pdl(k_step_pair_seq<L, ST, C, F, FO>, g, dim3(128), s, a, m);
         }
     }
     // FP64 (bound by a pipe that each SM has its own share of): blocks of 64 spread a small lattice more
     // evenly over the SMs (32^3: 512 blocks over 152 SMs instead of 256)
-    dim3 g, b;
-    lattice_grid(a.nx, a.ny, a.nzc, &g, &b, sizeof(ST) == 8 ? 64 : 128);
-    return launch_pdl(k_step<L, ST, C, F, FO>, g, b, s, a);
+    constexpr int T = sizeof(ST) == 8 ? 64 : 128;
+    const NodeMap m = node_grid<1>(a, T, &g);
+    return launch_pdl(k_step<L, ST, C, F, FO>, g, dim3(T), s, a, m);
 }
 
 template <class L, class ST, int C, int F>

@@ -9,14 +9,28 @@ namespace lbm {
 template <class R>
 struct StepArgs;
 
-// geometry of a lattice launch: blocks of `threads` (128) covering x (and several y rows when nx is small)
-inline void lattice_grid(int nx, int ny, int nz, dim3* grid, dim3* block, int threads = 128) {
-    int bx = nx <= 32 ? 32 : (nx <= 64 ? 64 : 128);
-    if (bx > threads) bx = threads;
-    const int by = threads / bx;
+// geometry of a lattice launch: 128-thread blocks covering x (and several y rows when nx is small)
+inline void lattice_grid(int nx, int ny, int nz, dim3* grid, dim3* block) {
+    const int bx = nx <= 32 ? 32 : (nx <= 64 ? 64 : 128);
+    const int by = 128 / bx;
     *block = dim3(bx, by, 1);
     *grid = dim3((nx + bx - 1) / bx, (ny + by - 1) / by, nz);
 }
+
+// floor(n / d) for 0 <= n < 2^31 as (n m) >> s
+struct FastDiv {
+    unsigned m, s;
+};
+inline FastDiv fast_div(unsigned d) {
+    unsigned l = 0;
+    while ((1ull << l) < d) ++l;
+    return {(unsigned)(((1ull << (31 + l)) + d - 1) / d), 31 + l};
+}
+#ifdef __CUDACC__
+__device__ __forceinline__ int div_fast(int n, FastDiv d) {
+    return (int)(((unsigned long long)(unsigned)n * d.m) >> d.s);
+}
+#endif
 
 // Programmatic dependent launch of a step (or adjoint step) kernel: consecutive steps overlap launch and block
 // scheduling with the previous step's tail (the kernel waits for the previous one before its
@@ -47,17 +61,8 @@ struct StreamCtl {
     int tiles_y;     // units per z plane: ceil(ny / rows)
     int first_step;  // 0; 1 only for the diagnostic that makes every dependency wait run out
     long long ring;  // 0: two buffers; else step k's buffers are the first ones shifted by k * ring elements
+    FastDiv row;     // thread positions per row: nx nodes, or nx / 2 pairs (filled by the launcher)
 };
-
-// floor(n / d) for 0 <= n < 2^31 as (n m) >> s
-struct FastDiv {
-    unsigned m, s;
-};
-inline FastDiv fast_div(unsigned d) {
-    unsigned l = 0;
-    while ((1ull << l) < d) ++l;
-    return {(unsigned)(((1ull << (31 + l)) + d - 1) / d), 31 + l};
-}
 
 constexpr int SUM_BLOCKS = 608;  // 4 blocks per SM on 152 SMs; partial rows in scratch
 

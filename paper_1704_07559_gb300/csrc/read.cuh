@@ -14,37 +14,13 @@
 
 namespace lbm {
 
-// One thread per node in node order over the computed planes, so that rows of any length fill the blocks.
-struct NodeMap {
-    FastDiv nx, ny;
-    int nodes;
-};
-template <class RS>
-inline NodeMap node_map(const StepArgs<RS>& a) {
-    return {fast_div((unsigned)a.nx), fast_div((unsigned)a.ny), a.nx * a.ny * a.nzc};
-}
-__device__ __forceinline__ int div_fast(int n, FastDiv d) {
-    return (int)(((unsigned long long)(unsigned)n * d.m) >> d.s);
-}
-template <class RS>
-__device__ __forceinline__ bool node_at(const StepArgs<RS>& a, const NodeMap& g, int& x, int& y, int& z) {
-    const unsigned t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= (unsigned)g.nodes) return false;
-    const int row = div_fast((int)t, g.nx);
-    x = (int)t - row * a.nx;
-    const int zz = div_fast(row, g.ny);
-    y = row - zz * a.ny;
-    z = zz + a.z0;
-    return true;
-}
-
 template <class L, class ST, int CLOSURE, int FORMULA, bool FORCE>
 __global__ void __launch_bounds__(128) k_strain(const StepArgs<typename Store<ST>::R> a, const NodeMap g) {
     using R = typename Store<ST>::R;
     pdl_wait();
     pdl_release();
     int x, y, z;
-    if (!node_at(a, g, x, y, z)) return;
+    if (!node_at<1>(a, g, x, y, z)) return;
     const int node = (z * a.ny + y) * a.nx + x;
     const long long N = (long long)a.nx * a.ny * a.nz;  // component offsets c*N exceed 2^31 on big grids
     R f[L::Q], P[L::NP], Dd[L::NP], F[3];
@@ -69,7 +45,7 @@ __global__ void __launch_bounds__(128) k_macro(const StepArgs<typename Store<ST>
     pdl_wait();
     pdl_release();
     int x, y, z;
-    if (!node_at(a, g, x, y, z)) return;
+    if (!node_at<1>(a, g, x, y, z)) return;
     const int node = (z * a.ny + y) * a.nx + x;
     const long long N = (long long)a.nx * a.ny * a.nz;
     R f[L::Q], P[L::NP], Dd[L::NP], F[3];
@@ -187,8 +163,8 @@ template <class L, class ST, int C, int F>
 cudaError_t launch_strain_cf(const StepArgs<typename Store<ST>::R>& a, int force, cudaStream_t s) {
     // FP64: blocks of 64, as the step
     constexpr int T = sizeof(ST) == 8 ? 64 : 128;
-    const NodeMap g = node_map(a);
-    const dim3 grid((unsigned)((g.nodes + (long long)T - 1) / T));
+    const NodeMap g = node_map<1>(a);
+    const dim3 grid((unsigned)((g.threads + (long long)T - 1) / T));
     return force ? launch_pdl(k_strain<L, ST, C, F, true>, grid, dim3(T), s, a, g)
                  : launch_pdl(k_strain<L, ST, C, F, false>, grid, dim3(T), s, a, g);
 }
@@ -215,8 +191,8 @@ cudaError_t launch_strain(const StepArgs<typename Store<ST>::R>& a, int closure,
 template <class L, class ST>
 cudaError_t launch_macro(const StepArgs<typename Store<ST>::R>& a, int formula, int force, cudaStream_t s) {
     constexpr int T = sizeof(ST) == 8 ? 64 : 128;
-    const NodeMap g = node_map(a);
-    const dim3 grid((unsigned)((g.nodes + (long long)T - 1) / T));
+    const NodeMap g = node_map<1>(a);
+    const dim3 grid((unsigned)((g.threads + (long long)T - 1) / T));
     if (formula == F_YU)
         return force ? launch_pdl(k_macro<L, ST, F_YU, true>, grid, dim3(T), s, a, g)
                      : launch_pdl(k_macro<L, ST, F_YU, false>, grid, dim3(T), s, a, g);

@@ -36,6 +36,7 @@
 #include <utility>
 
 #include "lattice.cuh"
+#include "launch.h"
 #include "power_law.h"
 
 
@@ -1352,6 +1353,49 @@ __device__ __forceinline__ void step_body(const StepArgs<typename Store<ST>::R>&
     sfor<Q>([&](auto i) { Store<ST>::st(static_cast<ST*>(a.dstp[CV(i)]) + ds + node, f[i] - out[i]); });
 }
 
+// Which node(s) a thread takes: PER x-adjacent nodes each (nx a multiple of PER), in node order over the
+// computed planes, so that rows of any length fill the blocks: with blocks cut at the row ends the step ran
+// (GLUPS, before -> now) FP32 200x150x97 channel 35.8 -> 40.6, 97x150x97 28.6 -> 37.1, 80^3 box 37.1 -> 45.9,
+// 301x301x199 39.0 -> 45.3, FP16 200x150x97 42.8 -> 50.9, 96^3 48.1 -> 63.8.  On rows that fill whole blocks
+// anyway (nx.m = 0) the grid gives x, y and z directly, without the two divisions.
+struct NodeMap {
+    FastDiv nx, ny;  // thread positions per row, rows per plane
+    int threads;     // thread positions in all
+};
+template <int PER, class RS>
+inline NodeMap node_map(const StepArgs<RS>& a) {
+    return {fast_div((unsigned)(a.nx / PER)), fast_div((unsigned)a.ny), a.nx / PER * a.ny * a.nzc};
+}
+template <int PER, class RS>
+__device__ __forceinline__ bool node_at(const StepArgs<RS>& a, const NodeMap& g, int& x, int& y, int& z) {
+    if (g.nx.m == 0) {
+        x = PER * (blockIdx.x * blockDim.x + threadIdx.x);
+        y = blockIdx.y;
+        z = blockIdx.z + a.z0;
+        return true;
+    }
+    const unsigned t = blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= (unsigned)g.threads) return false;
+    const int row = div_fast((int)t, g.nx), zz = div_fast(row, g.ny);
+    x = PER * (int)t - row * a.nx;
+    y = row - zz * a.ny;
+    z = zz + a.z0;
+    return true;
+}
+// the launch geometry of a map for blocks of `threads`
+template <int PER, class RS>
+inline NodeMap node_grid(const StepArgs<RS>& a, int threads, dim3* grid) {
+    NodeMap g = node_map<PER>(a);
+    const int row = a.nx / PER;
+    if (row % threads == 0) {
+        g.nx.m = 0;
+        *grid = dim3(row / threads, a.ny, a.nzc);
+    } else {
+        *grid = dim3((unsigned)((g.threads + (long long)threads - 1) / threads));
+    }
+    return g;
+}
+
 // One node per thread.  The bound names no minimum of resident blocks for the 3D lattices and
 // FP64: a minimum of one changes ptxas's register allocation (more registers, fewer resident
 // blocks).  FP32 D2Q9 is held to 16 blocks (32 registers, full occupancy; the power law spills up to 12
@@ -1363,13 +1407,12 @@ constexpr int step_min_blocks() {
 }
 
 template <class L, class ST, int CLOSURE, int FORMULA, bool FORCE>
-__global__ void __launch_bounds__(128, step_min_blocks<L, ST>()) k_step(const StepArgs<typename Store<ST>::R> a) {
+__global__ void __launch_bounds__(128, step_min_blocks<L, ST>())
+    k_step(const StepArgs<typename Store<ST>::R> a, const NodeMap g) {
     pdl_wait();     // the previous step's stores are complete and visible from here on
     pdl_release();  // every block has started: the next step may be scheduled into freed slots
-    const int x = blockIdx.x * blockDim.x + threadIdx.x;
-    const int y = blockIdx.y * blockDim.y + threadIdx.y;
-    const int z = blockIdx.z + a.z0;
-    if (x >= a.nx || y >= a.ny) return;
+    int x, y, z;
+    if (!node_at<1>(a, g, x, y, z)) return;
     typename Store<ST>::R f[L::Q];
     pull<L, ST>(a, x, y, z, f);
     step_body<L, ST, CLOSURE, FORMULA, FORCE>(a, f, (z * a.ny + y) * a.nx + x);

@@ -213,13 +213,12 @@ __device__ __forceinline__ void step_pair(const StepArgs<float>& a, const F2 (&f
 constexpr int PAIR_MIN_BLOCKS = 7;
 
 template <class L, class ST, int CLOSURE, int FORMULA, bool FORCE>
-__global__ void __launch_bounds__(128, PAIR_MIN_BLOCKS) k_step_pair_seq(const StepArgs<typename Store<ST>::R> a) {
+__global__ void __launch_bounds__(128, PAIR_MIN_BLOCKS)
+    k_step_pair_seq(const StepArgs<typename Store<ST>::R> a, const NodeMap g) {
     pdl_wait();
     pdl_release();
-    const int x = (blockIdx.x * blockDim.x + threadIdx.x) * 2;
-    const int y = blockIdx.y * blockDim.y + threadIdx.y;
-    const int z = blockIdx.z + a.z0;
-    if (x >= a.nx || y >= a.ny) return;
+    int x, y, z;
+    if (!node_at<2>(a, g, x, y, z)) return;
     F2 f2[L::Q];
     pull2<L, ST>(a, x, y, z, f2);
     step_pair<L, ST, CLOSURE, FORMULA, FORCE>(a, f2, (z * a.ny + y) * a.nx + x);
