@@ -26,6 +26,7 @@ struct lbm_ctx {
     long long N, stride;
     int elem_bytes;
     double rates[19];
+    double rates_n[19];  // s_k / |T_k|^2
     double force[3];
     lbm_params p;
     // bound resources
@@ -116,9 +117,8 @@ void fill_args(const lbm_ctx* c, lbm::StepArgs<R>* a) {
     a->nzc = c->nzc;
     a->stride = c->stride;
     for (int k = 0; k < 19; ++k) {
-        a->s[k] = R(k < c->q ? c->rates[k] : 0.0);
-        const int n2 = k >= c->q ? 1 : row_norm2(c->q, k);
-        a->skn[k] = R(k < c->q ? c->rates[k] / n2 : 0.0);
+        a->s[k] = R(c->rates[k]);
+        a->skn[k] = R(c->rates_n[k]);
     }
     for (int d = 0; d < 3; ++d) a->F[d] = R(c->force[d]);
     a->rho0 = R(c->p.rho0);
@@ -237,25 +237,17 @@ int stream_flag(lbm_ctx* c) {
     return LBM_OK;
 }
 
-// one step from src to dst through the right instantiation
-cudaError_t run_step(lbm_ctx* c, const void* src, void* dst) {
-    const int force = has_force(c) ? 1 : 0;
-    const Tag t = tag_of(c->q, c->p.precision);
-    if (c->p.precision == LBM_FP64) {
-        lbm::StepArgs<double> a;
-        fill_args(c, &a);
-        set_buffers(c, &a, src, dst);
-        switch (t) {
-            case T_D3Q19_F64: return lbm::step_d3q19_f64(a, c->p.closure, c->p.formula, force, c->stream);
-            case T_D3Q15_F64: return lbm::step_d3q15_f64(a, c->p.closure, c->p.formula, force, c->stream);
-            case T_D2Q9_F64: return lbm::step_d2q9_f64(a, c->p.closure, c->p.formula, force, c->stream);
-            default: return cudaErrorInvalidValue;
-        }
+// one step with the given arguments through the right instantiation
+cudaError_t launch_step(const lbm_ctx* c, const lbm::StepArgs<double>& a, int force) {
+    switch (tag_of(c->q, c->p.precision)) {
+        case T_D3Q19_F64: return lbm::step_d3q19_f64(a, c->p.closure, c->p.formula, force, c->stream);
+        case T_D3Q15_F64: return lbm::step_d3q15_f64(a, c->p.closure, c->p.formula, force, c->stream);
+        case T_D2Q9_F64: return lbm::step_d2q9_f64(a, c->p.closure, c->p.formula, force, c->stream);
+        default: return cudaErrorInvalidValue;
     }
-    lbm::StepArgs<float> a;
-    fill_args(c, &a);
-    set_buffers(c, &a, src, dst);
-    switch (t) {
+}
+cudaError_t launch_step(const lbm_ctx* c, const lbm::StepArgs<float>& a, int force) {
+    switch (tag_of(c->q, c->p.precision)) {
         case T_D3Q19_F32: return lbm::step_d3q19_f32(a, c->p.closure, c->p.formula, force, c->stream);
         case T_D3Q19_F16: return lbm::step_d3q19_f16(a, c->p.closure, c->p.formula, force, c->stream);
         case T_D3Q19_BF16: return lbm::step_d3q19_bf16(a, c->p.closure, c->p.formula, force, c->stream);
@@ -265,6 +257,37 @@ cudaError_t run_step(lbm_ctx* c, const void* src, void* dst) {
         case T_D2Q9_F32: return lbm::step_d2q9_f32(a, c->p.closure, c->p.formula, force, c->stream);
         default: return cudaErrorInvalidValue;
     }
+}
+
+// one step from src to dst
+template <class R>
+cudaError_t step_between(const lbm_ctx* c, const void* src, void* dst) {
+    lbm::StepArgs<R> a;
+    fill_args(c, &a);
+    set_buffers(c, &a, src, dst);
+    return launch_step(c, a, has_force(c) ? 1 : 0);
+}
+cudaError_t run_step(const lbm_ctx* c, const void* src, void* dst) {
+    return c->p.precision == LBM_FP64 ? step_between<double>(c, src, dst) : step_between<float>(c, src, dst);
+}
+
+// n steps from the current buffer, one launch each, from two sets of arguments filled once: a small
+// lattice's step is no longer than what the host does between two launches
+template <class R>
+cudaError_t step_by_step(lbm_ctx* c, int n, long long* launches) {
+    lbm::StepArgs<R> a[2];
+    fill_args(c, &a[0]);
+    a[1] = a[0];
+    set_buffers(c, &a[0], c->buf[0], c->buf[1]);
+    set_buffers(c, &a[1], c->buf[1], c->buf[0]);
+    const int force = has_force(c) ? 1 : 0;
+    for (int it = 0; it < n; ++it) {
+        cudaError_t e = launch_step(c, a[c->cur], force);
+        if (e != cudaSuccess) return e;
+        c->cur = 1 - c->cur;
+        ++*launches;
+    }
+    return cudaSuccess;
 }
 
 // S (and tau) of the state the next step sees, by `formula`
@@ -356,13 +379,8 @@ cudaError_t advance(lbm_ctx* c, int n, long long* launches) {
             ++*launches;
         }
     }
-    for (; it < n; ++it) {
-        cudaError_t e = run_step(c, c->buf[c->cur], c->buf[1 - c->cur]);
-        if (e != cudaSuccess) return e;
-        c->cur = 1 - c->cur;
-        ++*launches;
-    }
-    return cudaSuccess;
+    if (it == n) return cudaSuccess;
+    return c->p.precision == LBM_FP64 ? step_by_step<double>(c, n - it, launches) : step_by_step<float>(c, n - it, launches);
 }
 
 int check_bound(lbm_ctx* c) {
@@ -810,6 +828,7 @@ int lbm_create(lbm_ctx** out, int lattice, int nx, int ny, int nz, const double*
             return bad("rate range");
         }
         c->rates[k] = s;
+        c->rates_n[k] = s / row_norm2(c->q, k);
     }
     for (int d = 0; d < 3; ++d) c->force[d] = (force && d < c->d) ? force[d] : 0.0;
     for (int d = 0; d < 3; ++d)
