@@ -267,13 +267,12 @@ __global__ void __launch_bounds__(128) k_adjoint_step(const AdjArgs<typename Sto
 // accumulator, which other blocks of the launch wrote, are read through L2; the states are
 // read-only for the whole launch.
 template <class ST, int CLOSURE>
-__device__ __forceinline__ void adjoint_unit(const AdjArgs<typename Store<ST>::R>& a, FastDiv row, int z, int y0,
+__device__ __forceinline__ void adjoint_unit(const AdjArgs<typename Store<ST>::R>& a, const RowWalk& w, int z, int y0,
                                              int y1, long long es) {
     using R = typename Store<ST>::R;
     const long long N = (long long)a.st.nx * a.st.ny * a.st.nz;
-    const int n = (y1 - y0) * a.st.nx;  // in node order, as stream_unit
-    for (int t = threadIdx.x; t < n; t += blockDim.x) {
-        const int r = div_fast(t, row), y = y0 + r, x = t - r * a.st.nx;
+    const int r0 = div_fast(threadIdx.x, w.div);  // in node order, as stream_unit
+    for (int x = threadIdx.x - r0 * w.row, y = y0 + r0; y < y1;) {
         const int node = (z * a.st.ny + y) * a.st.nx + x;
         R p[19], F[3], lam[19], acc[3];
         pull<D3Q19, ST>(a.st, x, y, z, p, es);
@@ -289,6 +288,12 @@ __device__ __forceinline__ void adjoint_unit(const AdjArgs<typename Store<ST>::R
         node_backward<CLOSURE, true>(st, lam, Sb, R(0), a.st, mu, Fb);
         push(a, x, y, z, mu);
         for (int d = 0; d < 3; ++d) a.dF[d * N + node] = acc[d] + Fb[d];
+        x += w.dr;
+        y += w.dq;
+        if (x >= w.row) {
+            x -= w.row;
+            ++y;
+        }
     }
 }
 
@@ -300,9 +305,9 @@ __global__ void __launch_bounds__(128, 8) k_adjoint_stream(const AdjArgs<typenam
     stream_schedule(a0.st.ny, a0.st.nz, c, [&](int k, int z, int y0, int y1) {
         const long long es = -(long long)k * c.ring;
         if (k & 1)
-            adjoint_unit<ST, CLOSURE>(a1, c.row, z, y0, y1, es);
+            adjoint_unit<ST, CLOSURE>(a1, c.walk, z, y0, y1, es);
         else
-            adjoint_unit<ST, CLOSURE>(a0, c.row, z, y0, y1, es);
+            adjoint_unit<ST, CLOSURE>(a0, c.walk, z, y0, y1, es);
     });
 }
 

@@ -27,8 +27,10 @@ cudaError_t launch_form(const StepArgs<typename Store<ST>::R>& a, cudaStream_t s
     // FP64 (bound by a pipe that each SM has its own share of): blocks of 64 spread a small lattice more
     // evenly over the SMs (32^3: 512 blocks over 152 SMs instead of 256)
     constexpr int T = sizeof(ST) == 8 ? 64 : 128;
-    const NodeMap m = node_grid<1>(a, T, &g);
-    return launch_pdl(k_step<L, ST, C, F, FO>, g, dim3(T), s, a, m);
+    NodeMap m = node_grid<1>(a, T, &g);
+    dim3 b(T);
+    if constexpr (L::D == 2) lattice_grid(a.nx, a.ny, a.nzc, &g, &b);
+    return launch_pdl(k_step<L, ST, C, F, FO>, g, b, s, a, m);
 }
 
 template <class L, class ST, int C, int F>

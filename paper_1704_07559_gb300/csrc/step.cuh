@@ -1356,8 +1356,10 @@ __device__ __forceinline__ void step_body(const StepArgs<typename Store<ST>::R>&
 // Which node(s) a thread takes: PER x-adjacent nodes each (nx a multiple of PER), in node order over the
 // computed planes, so that rows of any length fill the blocks: with blocks cut at the row ends the step ran
 // (GLUPS, before -> now) FP32 200x150x97 channel 35.8 -> 40.6, 97x150x97 28.6 -> 37.1, 80^3 box 37.1 -> 45.9,
-// 301x301x199 39.0 -> 45.3, FP16 200x150x97 42.8 -> 50.9, 96^3 48.1 -> 63.8.  On rows that fill whole blocks
-// anyway (nx.m = 0) the grid gives x, y and z directly, without the two divisions.
+// 301x301x199 39.0 -> 45.3, FP16 200x150x97 42.8 -> 50.9, 96^3 48.1 -> 63.8.  Rows that leave at most a
+// sixteenth of their blocks' threads idle (nx.m = 0) keep a grid that gives x, y and z directly, without
+// the two divisions; D2Q9 steps, the lightest, always do (2000x1000 88.0 GLUPS, with either map chosen at
+// run time 86.0; 1000^2 in node order 92.1 against 97.4).
 struct NodeMap {
     FastDiv nx, ny;  // thread positions per row, rows per plane
     int threads;     // thread positions in all
@@ -1372,7 +1374,7 @@ __device__ __forceinline__ bool node_at(const StepArgs<RS>& a, const NodeMap& g,
         x = PER * (blockIdx.x * blockDim.x + threadIdx.x);
         y = blockIdx.y;
         z = blockIdx.z + a.z0;
-        return true;
+        return x < a.nx;
     }
     const unsigned t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= (unsigned)g.threads) return false;
@@ -1386,10 +1388,10 @@ __device__ __forceinline__ bool node_at(const StepArgs<RS>& a, const NodeMap& g,
 template <int PER, class RS>
 inline NodeMap node_grid(const StepArgs<RS>& a, int threads, dim3* grid) {
     NodeMap g = node_map<PER>(a);
-    const int row = a.nx / PER;
-    if (row % threads == 0) {
+    const int row = a.nx / PER, blocks = (row + threads - 1) / threads;
+    if ((long long)blocks * threads - row <= row / 16) {
         g.nx.m = 0;
-        *grid = dim3(row / threads, a.ny, a.nzc);
+        *grid = dim3(blocks, a.ny, a.nzc);
     } else {
         *grid = dim3((unsigned)((g.threads + (long long)threads - 1) / threads));
     }
@@ -1412,7 +1414,14 @@ __global__ void __launch_bounds__(128, step_min_blocks<L, ST>())
     pdl_wait();     // the previous step's stores are complete and visible from here on
     pdl_release();  // every block has started: the next step may be scheduled into freed slots
     int x, y, z;
-    if (!node_at<1>(a, g, x, y, z)) return;
+    if constexpr (L::D == 2) {
+        x = blockIdx.x * blockDim.x + threadIdx.x;
+        y = blockIdx.y * blockDim.y + threadIdx.y;
+        z = 0;
+        if (x >= a.nx || y >= a.ny) return;
+    } else {
+        if (!node_at<1>(a, g, x, y, z)) return;
+    }
     typename Store<ST>::R f[L::Q];
     pull<L, ST>(a, x, y, z, f);
     step_body<L, ST, CLOSURE, FORMULA, FORCE>(a, f, (z * a.ny + y) * a.nx + x);

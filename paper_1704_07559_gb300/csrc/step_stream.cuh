@@ -70,23 +70,31 @@ __device__ __noinline__ static bool wait_count(const int* flag, int want, int* e
 
 // One unit: rows [y0, y1) of plane z, one node per thread (PAIR false) or two x-adjacent nodes
 // per thread in packed pair arithmetic (PAIR true, nx even), in node order, so that rows of any length keep
-// the block's threads busy; `row` divides a position by the positions per row.  es / ds shift the source /
-// destination populations by that many elements (ring launches; one node per thread only).
+// the block's threads busy.  es / ds shift the source / destination populations by that many elements (ring
+// launches; one node per thread only).
 template <class L, class ST, int CLOSURE, int FORMULA, bool FORCE, bool PAIR>
-__device__ __forceinline__ void stream_unit(const StepArgs<typename Store<ST>::R>& a, FastDiv row, int z, int y0, int y1,
+__device__ __forceinline__ void stream_unit(const StepArgs<typename Store<ST>::R>& a, const RowWalk& w, int z, int y0, int y1,
                                             long long es = 0, long long ds = 0) {
     using R = typename Store<ST>::R;
-    const int n = (y1 - y0) * (PAIR ? a.nx / 2 : a.nx);
-    for (int t = threadIdx.x; t < n; t += blockDim.x) {
-        const int r = div_fast(t, row), y = y0 + r, x = (PAIR ? 2 * t : t) - r * a.nx;
+    const int r0 = div_fast(threadIdx.x, w.div);
+    for (int p = threadIdx.x - r0 * w.row, y = y0 + r0; y < y1;) {
+        const int x = PAIR ? 2 * p : p;
         if constexpr (PAIR) {
-            F2 f2[L::Q];
-            pull2<L, ST, true>(a, x, y, z, f2);
-            step_pair<L, ST, CLOSURE, FORMULA, FORCE>(a, f2, (z * a.ny + y) * a.nx + x);
+            if (x < a.nx) {
+                F2 f2[L::Q];
+                pull2<L, ST, true>(a, x, y, z, f2);
+                step_pair<L, ST, CLOSURE, FORMULA, FORCE>(a, f2, (z * a.ny + y) * a.nx + x);
+            }
         } else {
             R f[L::Q];
             pull<L, ST, true>(a, x, y, z, f, es);
             step_body<L, ST, CLOSURE, FORMULA, FORCE>(a, f, (z * a.ny + y) * a.nx + x, ds);
+        }
+        p += w.dr;
+        y += w.dq;
+        if (p >= w.row) {
+            p -= w.row;
+            ++y;
         }
     }
 }
@@ -156,9 +164,9 @@ __device__ __forceinline__ void stream_steps(const StepArgs<typename Store<ST>::
                                              const StepArgs<typename Store<ST>::R>& a1, const StreamCtl& c) {
     stream_schedule(a0.ny, a0.nz, c, [&](int k, int z, int y0, int y1) {
         if (k & 1)
-            stream_unit<L, ST, CLOSURE, FORMULA, FORCE, PAIR>(a1, c.row, z, y0, y1);
+            stream_unit<L, ST, CLOSURE, FORMULA, FORCE, PAIR>(a1, c.walk, z, y0, y1);
         else
-            stream_unit<L, ST, CLOSURE, FORMULA, FORCE, PAIR>(a0, c.row, z, y0, y1);
+            stream_unit<L, ST, CLOSURE, FORMULA, FORCE, PAIR>(a0, c.walk, z, y0, y1);
     });
 }
 
@@ -197,7 +205,7 @@ __global__ void __launch_bounds__(128, FORMULA == F_YU ? 9 : 7)
     k_step_stream_ring(const StepArgs<typename Store<ST>::R> a, const StreamCtl c) {
     stream_schedule(a.ny, a.nz, c, [&](int k, int z, int y0, int y1) {
         const long long sh = k * c.ring;
-        stream_unit<L, ST, CLOSURE, FORMULA, FORCE, false>(a, c.row, z, y0, y1, sh, sh);
+        stream_unit<L, ST, CLOSURE, FORMULA, FORCE, false>(a, c.walk, z, y0, y1, sh, sh);
     });
 }
 
@@ -247,7 +255,7 @@ cudaError_t launch_stream_form(const StepArgs<typename Store<ST>::R>& a0, const 
         if (a0.nx % 2 == 0) {
             static const int resident = resident_blocks(k_step_stream_pair<L, ST, C, F, FO>);
             if (!pick_units(c, a0.ny, a0.nz, resident, &u) && !force_stream) return cudaErrorNotSupported;
-            u.row = fast_div((unsigned)(a0.nx / 2));
+            u.walk = row_walk(a0.nx / 2, true);
             const long long total = (long long)a0.nz * u.tiles_y * u.steps;
             if (total >= (1LL << 31) || u.steps < 1) return cudaErrorInvalidValue;
             const int grid = (int)(total < resident ? total : resident);
@@ -259,7 +267,7 @@ cudaError_t launch_stream_form(const StepArgs<typename Store<ST>::R>& a0, const 
     }
     static const int resident = resident_blocks(k_step_stream<L, ST, C, F, FO>);
     if (!pick_units(c, a0.ny, a0.nz, resident, &u) && !force_stream) return cudaErrorNotSupported;
-    u.row = fast_div((unsigned)a0.nx);
+    u.walk = row_walk(a0.nx, false);
     const long long total = (long long)a0.nz * u.tiles_y * u.steps;
     if (total >= (1LL << 31) || u.steps < 1) return cudaErrorInvalidValue;
     const int grid = (int)(total < resident ? total : resident);
@@ -277,7 +285,7 @@ cudaError_t launch_stream_ring_form(const StepArgs<typename Store<ST>::R>& a, co
     static const int resident = resident_blocks(k_step_stream_ring<L, ST, C, F, FO>);
     StreamCtl u;
     if (!pick_units(c, a.ny, a.nz, resident, &u) && !force_stream) return cudaErrorNotSupported;
-    u.row = fast_div((unsigned)a.nx);
+    u.walk = row_walk(a.nx, false);
     const long long total = (long long)a.nz * u.tiles_y * u.steps;
     if (total >= (1LL << 31) || u.steps < 1) return cudaErrorInvalidValue;
     const int grid = (int)(total < resident ? total : resident);
