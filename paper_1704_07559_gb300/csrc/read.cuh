@@ -20,7 +20,7 @@ __global__ void __launch_bounds__(128) k_strain(const StepArgs<typename Store<ST
     pdl_wait();
     pdl_release();
     int x, y, z;
-    if (!node_at<1>(a, g, x, y, z)) return;
+    if (!node_in_order<1>(a, g, x, y, z)) return;
     const int node = (z * a.ny + y) * a.nx + x;
     const long long N = (long long)a.nx * a.ny * a.nz;  // component offsets c*N exceed 2^31 on big grids
     R f[L::Q], P[L::NP], Dd[L::NP], F[3];
@@ -45,7 +45,7 @@ __global__ void __launch_bounds__(128) k_macro(const StepArgs<typename Store<ST>
     pdl_wait();
     pdl_release();
     int x, y, z;
-    if (!node_at<1>(a, g, x, y, z)) return;
+    if (!node_in_order<1>(a, g, x, y, z)) return;
     const int node = (z * a.ny + y) * a.nx + x;
     const long long N = (long long)a.nx * a.ny * a.nz;
     R f[L::Q], P[L::NP], Dd[L::NP], F[3];

@@ -1313,7 +1313,7 @@ __device__ __forceinline__ void step_body(const StepArgs<typename Store<ST>::R>&
     // every collision increment D_k = (s_k mn_k - TF_k) / |T_k|^2 that does not involve an unknown
     // viscous rate is finished before the closure, so only the viscous moments (and their force terms)
     // stay live across the fixed point
-    constexpr bool KNOWN = rates_known<CLOSURE, FORMULA>();
+    constexpr bool KNOWN = CLOSURE == CL_NEWTON;  // every rate given: S is not needed
     R Dk[Q], tv[Q];
     sfor<Q>([&](auto k) {
         constexpr double inv_n = 1.0 / norm2<L>(CV(k));
@@ -1356,10 +1356,9 @@ __device__ __forceinline__ void step_body(const StepArgs<typename Store<ST>::R>&
 // Which node(s) a thread takes: PER x-adjacent nodes each (nx a multiple of PER), in node order over the
 // computed planes, so that rows of any length fill the blocks: with blocks cut at the row ends the step ran
 // (GLUPS, before -> now) FP32 200x150x97 channel 35.8 -> 40.6, 97x150x97 28.6 -> 37.1, 80^3 box 37.1 -> 45.9,
-// 301x301x199 39.0 -> 45.3, FP16 200x150x97 42.8 -> 50.9, 96^3 48.1 -> 63.8.  Rows that leave at most a
-// sixteenth of their blocks' threads idle (nx.m = 0) keep a grid that gives x, y and z directly, without
-// the two divisions; D2Q9 steps, the lightest, always do (2000x1000 88.0 GLUPS, with either map chosen at
-// run time 86.0; 1000^2 in node order 92.1 against 97.4).
+// 301x301x199 39.0 -> 45.3, FP16 200x150x97 42.8 -> 50.9, 96^3 48.1 -> 63.8.  Where rows fill whole blocks
+// anyway (nx.m = 0) the grid gives x, y and z directly, without the two divisions; the FP32 and FP64 steps
+// are built for each map, since choosing at run time cost them up to 8% (121x89x38 channel).
 struct NodeMap {
     FastDiv nx, ny;  // thread positions per row, rows per plane
     int threads;     // thread positions in all
@@ -1369,13 +1368,14 @@ inline NodeMap node_map(const StepArgs<RS>& a) {
     return {fast_div((unsigned)(a.nx / PER)), fast_div((unsigned)a.ny), a.nx / PER * a.ny * a.nzc};
 }
 template <int PER, class RS>
-__device__ __forceinline__ bool node_at(const StepArgs<RS>& a, const NodeMap& g, int& x, int& y, int& z) {
-    if (g.nx.m == 0) {
-        x = PER * (blockIdx.x * blockDim.x + threadIdx.x);
-        y = blockIdx.y;
-        z = blockIdx.z + a.z0;
-        return x < a.nx;
-    }
+__device__ __forceinline__ bool node_in_grid(const StepArgs<RS>& a, int& x, int& y, int& z) {
+    x = PER * (blockIdx.x * blockDim.x + threadIdx.x);
+    y = blockIdx.y * blockDim.y + threadIdx.y;
+    z = blockIdx.z + a.z0;
+    return x < a.nx && y < a.ny;
+}
+template <int PER, class RS>
+__device__ __forceinline__ bool node_in_order(const StepArgs<RS>& a, const NodeMap& g, int& x, int& y, int& z) {
     const unsigned t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= (unsigned)g.threads) return false;
     const int row = div_fast((int)t, g.nx), zz = div_fast(row, g.ny);
@@ -1384,12 +1384,17 @@ __device__ __forceinline__ bool node_at(const StepArgs<RS>& a, const NodeMap& g,
     z = zz + a.z0;
     return true;
 }
-// the launch geometry of a map for blocks of `threads`
 template <int PER, class RS>
-inline NodeMap node_grid(const StepArgs<RS>& a, int threads, dim3* grid) {
+__device__ __forceinline__ bool node_at(const StepArgs<RS>& a, const NodeMap& g, int& x, int& y, int& z) {
+    return g.nx.m == 0 ? node_in_grid<PER>(a, x, y, z) : node_in_order<PER>(a, g, x, y, z);
+}
+// the launch geometry of a map for blocks of `threads`; rows that waste at most 1/waste of themselves in
+// idle threads (0: none) count as filling their blocks
+template <int PER, class RS>
+inline NodeMap node_grid(const StepArgs<RS>& a, int threads, int waste, dim3* grid) {
     NodeMap g = node_map<PER>(a);
     const int row = a.nx / PER, blocks = (row + threads - 1) / threads;
-    if ((long long)blocks * threads - row <= row / 16) {
+    if ((long long)blocks * threads - row <= (waste ? row / waste : 0)) {
         g.nx.m = 0;
         *grid = dim3(blocks, a.ny, a.nzc);
     } else {
@@ -1408,20 +1413,13 @@ constexpr int step_min_blocks() {
     return (L::Q == 9 && sizeof(ST) == 4) ? 16 : 0;
 }
 
-template <class L, class ST, int CLOSURE, int FORMULA, bool FORCE>
+template <class L, class ST, int CLOSURE, int FORMULA, bool FORCE, bool GRID>
 __global__ void __launch_bounds__(128, step_min_blocks<L, ST>())
     k_step(const StepArgs<typename Store<ST>::R> a, const NodeMap g) {
     pdl_wait();     // the previous step's stores are complete and visible from here on
     pdl_release();  // every block has started: the next step may be scheduled into freed slots
     int x, y, z;
-    if constexpr (L::D == 2) {
-        x = blockIdx.x * blockDim.x + threadIdx.x;
-        y = blockIdx.y * blockDim.y + threadIdx.y;
-        z = 0;
-        if (x >= a.nx || y >= a.ny) return;
-    } else {
-        if (!node_at<1>(a, g, x, y, z)) return;
-    }
+    if (!(GRID ? node_in_grid<1>(a, x, y, z) : node_in_order<1>(a, g, x, y, z))) return;
     typename Store<ST>::R f[L::Q];
     pull<L, ST>(a, x, y, z, f);
     step_body<L, ST, CLOSURE, FORMULA, FORCE>(a, f, (z * a.ny + y) * a.nx + x);

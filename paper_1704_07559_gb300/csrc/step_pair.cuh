@@ -41,22 +41,16 @@ __device__ __forceinline__ V2& operator+=(V2& a, V2 b) { return a = a + b; }
 __device__ __forceinline__ V2& operator-=(V2& a, V2 b) { return a = a - b; }
 __device__ __forceinline__ V2 fma(V2 a, V2 b, V2 c) { return V2(__ffma2_rn(a.v, b.v, c.v)); }
 
-// Smagorinsky / Newtonian closure for the pair: the quadratic form of |S|^2 in s = 1/tau is formed
-// for both lanes at once, then each lane runs the scalar fixed point of step.cuh.
+// Smagorinsky closure for the pair: the quadratic form of |S|^2 in s = 1/tau is formed for both lanes at
+// once, then each lane runs the scalar fixed point of step.cuh.
 template <class L, int CLOSURE>
-__device__ __forceinline__ V2 solve_tau_pair(const V2 (&A)[L::NS], const V2 (&B)[L::NS], const StepArgs<float>& a,
-                                            V2& snu) {
-    static_assert(CLOSURE == CL_NEWTON || CLOSURE == CL_SMAG, "16-bit storage builds these closures");
-    if constexpr (CLOSURE == CL_NEWTON) {
-        snu = V2(a.s[L::NU0]);
-        return V2(a.tau0);
-    } else {
-        const V2 qa = strain_dot<L>(A, A), qb2 = V2(2.0f) * strain_dot<L>(A, B), qc = strain_dot<L>(B, B);
-        const float t0 = tau_fixed_point<CLOSURE>(qa.lo(), qb2.lo(), qc.lo(), a);
-        const float t1 = tau_fixed_point<CLOSURE>(qa.hi(), qb2.hi(), qc.hi(), a);
-        snu = V2(c_rcp(t0), c_rcp(t1));
-        return V2(t0, t1);
-    }
+__device__ __forceinline__ void solve_tau_pair(const V2 (&A)[L::NS], const V2 (&B)[L::NS], const StepArgs<float>& a,
+                                              V2& snu) {
+    static_assert(CLOSURE == CL_SMAG, "16-bit storage builds this closure and fixed rates");
+    const V2 qa = strain_dot<L>(A, A), qb2 = V2(2.0f) * strain_dot<L>(A, B), qc = strain_dot<L>(B, B);
+    const float t0 = tau_fixed_point<CLOSURE>(qa.lo(), qb2.lo(), qc.lo(), a);
+    const float t1 = tau_fixed_point<CLOSURE>(qa.hi(), qb2.hi(), qc.hi(), a);
+    snu = V2(c_rcp(t0), c_rcp(t1));
 }
 
 // One step of the pair (node, node + 1) from its pulled populations: the step_body arithmetic on
@@ -127,22 +121,24 @@ __device__ __forceinline__ void step_pair(const StepArgs<float>& a, const F2 (&f
                     // the rate-independent part of G_k: (m_k + TF_k) / |T_k|^2, less s_k mn_k / |T_k|^2
                     // unless k is viscous
                     const R base = has_tf ? cst<R>(inv_n) * (m[k] + TF[k]) : cst<R>(inv_n) * m[k];
-                    if constexpr (L::viscous(CV(k)))
+                    if constexpr (L::viscous(CV(k)) && CLOSURE != CL_NEWTON)
                         G[k] = base;
                     else
                         G[k] = fma(R(-a.skn[k]), mn[k], base);
                 }
             });
         }
-        R A[NS], B[NS];
-        Eq<L>::yu_split(mn, R(a.s[1] * float(Eq<L>::YU_A)) * ir0, ir0, A, B);
-        solve_tau_pair<L, CLOSURE>(A, B, a, snu);
-        sfor<Q>([&](auto k) {
-            if constexpr (L::viscous(CV(k))) {
-                constexpr double inv_n = 1.0 / norm2<L>(CV(k));
-                G[k] = fma(-(snu * cst<R>(inv_n)), mn[k], G[k]);
-            }
-        });
+        if constexpr (CLOSURE != CL_NEWTON) {
+            R A[NS], B[NS];
+            Eq<L>::yu_split(mn, R(a.s[1] * float(Eq<L>::YU_A)) * ir0, ir0, A, B);
+            solve_tau_pair<L, CLOSURE>(A, B, a, snu);
+            sfor<Q>([&](auto k) {
+                if constexpr (L::viscous(CV(k))) {
+                    constexpr double inv_n = 1.0 / norm2<L>(CV(k));
+                    G[k] = fma(-(snu * cst<R>(inv_n)), mn[k], G[k]);
+                }
+            });
+        }
     } else {
         // Chai route: the non-equilibrium distributions f - f_eq + Fbar/2 (opposite-pair form), their
         // moments mn = T fn, and S from them with the contraction folded into T^-1 (chai_contract).
@@ -185,21 +181,14 @@ __device__ __forceinline__ void step_pair(const StepArgs<float>& a, const F2 (&f
                     G[k] = fma(cst<R>(inv_n), base, -Dn[k]);
             });
         }
-        if constexpr (CLOSURE == CL_NEWTON) {
-            // each viscous rate as given; with fixed rates S is a read-out only, not needed by the step
-            sfor<Q>([&](auto k) {
-                if constexpr (L::viscous(CV(k))) G[k] = fma(R(-a.s[k]), Dn[k], G[k]);
-            });
-        } else {
-            const R kS = R(-1.5f) * ir0;
-            R A[NS], B[NS];
-            chai_contract<L>(Dn, kS, [](int k) { return !L::conserved(k) && !L::viscous(k); }, A);
-            chai_contract<L>(Dn, kS, [](int k) { return L::viscous(k); }, B);
-            solve_tau_pair<L, CLOSURE>(A, B, a, snu);
-            sfor<Q>([&](auto k) {
-                if constexpr (L::viscous(CV(k))) G[k] = fma(-snu, Dn[k], G[k]);
-            });
-        }
+        const R kS = R(-1.5f) * ir0;
+        R A[NS], B[NS];
+        chai_contract<L>(Dn, kS, [](int k) { return !L::conserved(k) && !L::viscous(k); }, A);
+        chai_contract<L>(Dn, kS, [](int k) { return L::viscous(k); }, B);
+        solve_tau_pair<L, CLOSURE>(A, B, a, snu);
+        sfor<Q>([&](auto k) {
+            if constexpr (L::viscous(CV(k))) G[k] = fma(-snu, Dn[k], G[k]);
+        });
     }
     R fs[Q];
     Xf<L>::template backward<mask_all<L>()>(G, fs);
