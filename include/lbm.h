@@ -191,7 +191,9 @@ int lbm_step(lbm_ctx* ctx, int n);
  *                         more units (a z plane times a band of y rows of about 1024-4096 nodes)
  *                         than the GPU holds resident blocks; one launch per step otherwise (the
  *                         default).  On larger lattices, and on D2Q9 lattices, a step boundary
- *                         costs less than the multi-step launch's synchronisation.
+ *                         costs less than the multi-step launch's synchronisation.  FP32 D2Q9
+ *                         lattices (not with the lagged closure, and with the power law up to 2^19
+ *                         nodes) run four steps per launch in shared-memory tiles instead.
  *  LBM_SCHEDULE_PER_STEP  one launch per step.
  *  LBM_SCHEDULE_STREAM    several steps per launch wherever the storage allows it (not FP64),
  *                         whatever the lattice size.

@@ -34,7 +34,11 @@ cudaError_t launch_form(const StepArgs<typename Store<ST>::R>& a, cudaStream_t s
         lattice_grid(a.nx, a.ny, a.nzc, &g, &b);
         return launch_pdl(k_step<L, ST, C, F, FO, true>, g, b, s, a, NodeMap{});
     } else {
-        const NodeMap m = node_grid<1>(a, T, 0, &g);
+        // rows that nearly fill their blocks keep the plain grid only where both buffers stay in L2 (121x89x38,
+        // 62 MB: 38.6 against 36.5 GLUPS); from HBM blocks that start off a 128-byte line cost more than the
+        // two divisions (250x150x97: 39.6 against 42.5)
+        const bool in_l2 = 2LL * L::Q * a.stride * (int)sizeof(ST) <= (64LL << 20);
+        const NodeMap m = node_grid<1>(a, T, in_l2 ? 16 : 0, &g);
         return m.nx.m == 0 ? launch_pdl(k_step<L, ST, C, F, FO, true>, g, dim3(T), s, a, m)
                            : launch_pdl(k_step<L, ST, C, F, FO, false>, g, dim3(T), s, a, m);
     }

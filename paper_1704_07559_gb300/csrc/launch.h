@@ -51,11 +51,11 @@ inline RowWalk row_walk(int row, bool fill) {
 // scheduling with the previous step's tail (the kernel waits for the previous one before its
 // first load).
 template <class K, class... A>
-cudaError_t launch_pdl(K kernel, dim3 g, dim3 b, cudaStream_t s, const A&... a) {
+cudaError_t launch_pdl_smem(K kernel, dim3 g, dim3 b, int smem, cudaStream_t s, const A&... a) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = g;
     cfg.blockDim = b;
-    cfg.dynamicSmemBytes = 0;
+    cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -63,6 +63,10 @@ cudaError_t launch_pdl(K kernel, dim3 g, dim3 b, cudaStream_t s, const A&... a) 
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     return cudaLaunchKernelEx(&cfg, kernel, a...);
+}
+template <class K, class... A>
+cudaError_t launch_pdl(K kernel, dim3 g, dim3 b, cudaStream_t s, const A&... a) {
+    return launch_pdl_smem(kernel, g, b, 0, s, a...);
 }
 
 // Several steps in one launch (step_stream.cuh): the library-owned synchronisation words and the
@@ -119,6 +123,10 @@ LBM_DECLARE_STREAM_ENTRY(d3q15_f16, float)
 LBM_DECLARE_STREAM_ENTRY(d3q15_bf16, float)
 LBM_DECLARE_STREAM_ENTRY(d2q9_f32, float)
 #undef LBM_DECLARE_STREAM_ENTRY
+// BLOCK_STEPS steps per launch in shared-memory tiles (step_block.cuh); cudaErrorNotSupported where it does
+// not apply or pay, the caller then steps one by one
+constexpr int BLOCK_STEPS = 4;
+cudaError_t block_d2q9_f32(const StepArgs<float>& a, int closure, int formula, int force, cudaStream_t s);
 // ring launches (each step writes a buffer of its own): D3Q19 FP32, Newtonian and Smagorinsky
 cudaError_t stream_ring_d3q19_f32(const StepArgs<float>& a, const StreamCtl& c, int closure, int formula, int force,
                                   int force_stream, cudaStream_t s);

@@ -1290,12 +1290,11 @@ __device__ __forceinline__ void strain_split(const StepArgs<RS>& a, const R (&mn
 }
 
 // Everything of a step after the pull, for the node `node`: moments, strain rate by the chosen route,
-// closure, relaxation, force, and the store of f*.  ds shifts the populations' destination by that many
-// elements (a launch that writes each step to its own buffer of a ring); the pull's es does the same for
-// the source.
-template <class L, class ST, int CLOSURE, int FORMULA, bool FORCE>
-__device__ __forceinline__ void step_body(const StepArgs<typename Store<ST>::R>& a, typename Store<ST>::R (&f)[L::Q],
-                                          int node, long long ds = 0) {
+// closure, relaxation, force; sink(i, v) takes f*_i.  (With fixed rates a step needs no S, so one kernel,
+// the Yu route's, steps Newtonian lattices of either formula, each viscous moment with its own rate.)
+template <class L, class ST, int CLOSURE, int FORMULA, bool FORCE, class Sink>
+__device__ __forceinline__ void collide(const StepArgs<typename Store<ST>::R>& a, typename Store<ST>::R (&f)[L::Q],
+                                        int node, Sink&& sink) {
     using R = typename Store<ST>::R;
     constexpr int Q = L::Q, NS = L::NS, NP = L::NP;
 
@@ -1350,7 +1349,17 @@ __device__ __forceinline__ void step_body(const StepArgs<typename Store<ST>::R>&
     // f*_i = f_i - out_i; with a force, the conserved moments 3, 5, 7 (D2Q9: 3, 5) carry -TF_k; TF_0 = 0
     R out[Q];
     Xf<L>::template backward<FORCE ? mask_all_but_density<L>() : mask_nonconserved<L>()>(Dk, out);
-    sfor<Q>([&](auto i) { Store<ST>::st(static_cast<ST*>(a.dstp[CV(i)]) + ds + node, f[i] - out[i]); });
+    sfor<Q>([&](auto i) { sink(i, f[i] - out[i]); });
+}
+
+// The collision with f* stored at the node.  ds shifts the populations' destination by that many elements (a
+// launch that writes each step to its own buffer of a ring); the pull's es does the same for the source.
+template <class L, class ST, int CLOSURE, int FORMULA, bool FORCE>
+__device__ __forceinline__ void step_body(const StepArgs<typename Store<ST>::R>& a, typename Store<ST>::R (&f)[L::Q],
+                                          int node, long long ds = 0) {
+    collide<L, ST, CLOSURE, FORMULA, FORCE>(a, f, node, [&](auto i, auto v) {
+        Store<ST>::st(static_cast<ST*>(a.dstp[CV(i)]) + ds + node, v);
+    });
 }
 
 // Which node(s) a thread takes: PER x-adjacent nodes each (nx a multiple of PER), in node order over the

@@ -1,0 +1,130 @@
+// step_block.cuh -- BLOCK_STEPS steps of a D2Q9 lattice per launch, tile by tile in shared memory.
+//
+// One step per launch reads and writes every population once (72 B a node in FP32): from HBM that bounds large
+// lattices (4096^2 at 95 GLUPS, the copy bandwidth), and a small lattice's step takes 3 us however little it
+// computes (256^2 at 21.5 GLUPS).  Here a block owns BW x BH nodes and advances them 4 steps in one launch: the
+// first step pulls from global memory and computes the tile with a margin of 3 nodes, each following step
+// pulls from shared memory and computes a margin one node narrower, and the last one writes the tile's
+// nodes to the destination buffer.  Margins are computed by every tile that needs them, so no block waits for
+// another; a margin ends at a wall, where the pull reflects the node's own populations.  Every node update is
+// the one-step kernel's, so the state equals one launch per step bit for bit.
+//
+// Tile: 32 x 20, so that the first step's 38 x 26 nodes take one pass of 1024 threads (64 registers; 1.27 node
+// updates computed per one kept); 32 x 16 (1.31) where 32 x 20 leaves SMs without a tile.  Measured (Newtonian
+// Yu, GLUPS per step launch / 32x16 / 32x20): 256^2 21.5 / 38.6 / 36.5, 512^2 56.9 / 72.7 / 75.8, 1000^2 98.9 /
+// 104 / 110, 4096^2 95.3 / 122 / 131; 256 threads (several passes a step, few warps) 22 at 256^2, 110 at 4096^2;
+// 64x32 120 at 4096^2, 6 steps 112, 2 steps 103 (32x16).  Smagorinsky 4096^2 94 / 98 / 105, deviatoric Chai 95 /
+// 106 / 112.  The power law is bound by its sweeps, which margins repeat: 512^2 42.1 / 48.7 / 51.8 but 1000^2
+// 70.2 / 63.5 / 67.2 and 4096^2 84 / 72 / 77, so it takes this form up to 2^19 nodes only.
+#pragma once
+
+#include "launch.h"
+#include "step.cuh"
+
+namespace lbm {
+
+constexpr int BW = 32, BLOCK_THREADS = 1024;
+constexpr int BM = BLOCK_STEPS - 1;   // margin of the first step
+constexpr int SW = BW + 2 * BM;       // width of the shared tile
+// its height and its size, for tiles of BH rows
+constexpr int tile_rows(int BH) { return BH + 2 * BM; }
+constexpr int block_smem(int BH) { return 2 * 9 * SW * tile_rows(BH) * (int)sizeof(float); }
+
+// Pull of the node (x, y) at tile position t of the shared populations s (population i at i * PITCH): periodic
+// neighbours lie beside it in the tile, populations from behind a wall come from the node itself as in
+// pull_general.
+template <class L, int PITCH>
+__device__ __forceinline__ void pull_tile(const StepArgs<float>& a, const float* s, int t, int x, int y,
+                                          float (&f)[L::Q]) {
+    const int w = a.wall_mask;
+    const bool xl = (w & 1) && x == 0, xh = (w & 2) && x == a.nx - 1, yl = (w & 4) && y == 0,
+               yh = (w & 8) && y == a.ny - 1;
+    if (!(xl || xh || yl || yh)) {
+        sfor<L::Q>([&](auto i) {
+            f[i] = s[CV(i) * PITCH + t - L::c(CV(i), 0) - L::c(CV(i), 1) * SW];
+        });
+        return;
+    }
+    sfor<L::Q>([&](auto i) {
+        constexpr int cx = L::c(CV(i), 0), cy = L::c(CV(i), 1);
+        const bool ox = (cx > 0 && xl) || (cx < 0 && xh), oy = (cy > 0 && yl) || (cy < 0 && yh);
+        if (!ox && !oy) {
+            f[i] = s[CV(i) * PITCH + t - cx - cy * SW];
+        } else {
+            float v = s[opp<L>(CV(i)) * PITCH + t];
+            const int face = ox ? (cx > 0 ? 0 : 1) : (cy > 0 ? 2 : 3);
+            if (ox != oy && ((a.lid_mask >> face) & 1)) {
+                const float cu = float(cx) * a.lid[face][0] + float(cy) * a.lid[face][1] + 0.0f * a.lid[face][2];
+                v += float(double(6 * L::wnum(CV(i))) / L::WDEN) * a.rho0 * cu;
+            }
+            f[i] = v;
+        }
+    });
+}
+
+// position p of an axis of n nodes: wrapped on a periodic axis, as it is on an axis with walls
+__device__ __forceinline__ int wrap_pos(int p, int n, bool walls) {
+    if (walls) return p;
+    while (p < 0) p += n;
+    while (p >= n) p -= n;
+    return p;
+}
+
+template <class L, int CLOSURE, int FORMULA, bool FORCE, int BH>
+__global__ void __launch_bounds__(BLOCK_THREADS) k_step_block(const StepArgs<float> a) {
+    constexpr int SH = tile_rows(BH), PITCH = SW * SH;
+    extern __shared__ float sm[];
+    pdl_wait();
+    pdl_release();
+    const int ox = blockIdx.x * BW - BM, oy = blockIdx.y * BH - BM;
+    const bool wx = (a.wall_mask & 3) != 0, wy = (a.wall_mask & 12) != 0;
+    sfor<BLOCK_STEPS>([&](auto k) {
+        // step k computes the tile less k nodes on each side of the shared area
+        constexpr int W = SW - 2 * CV(k), H = SH - 2 * CV(k);
+        constexpr bool FIRST = CV(k) == 0, LAST = CV(k) == BLOCK_STEPS - 1;
+        const float* from = sm + (CV(k) & 1 ? 0 : 1) * 9 * PITCH;
+        float* to = sm + (CV(k) & 1) * 9 * PITCH;
+        for (int t = threadIdx.x; t < W * H; t += BLOCK_THREADS) {
+            const int ly = t / W + CV(k), lx = t - (t / W) * W + CV(k);
+            const int x = wrap_pos(ox + lx, a.nx, wx), y = wrap_pos(oy + ly, a.ny, wy);
+            bool mine = x >= 0 && x < a.nx && y >= 0 && y < a.ny;  // false only beyond a wall
+            if (LAST) mine = mine && ox + lx < a.nx && oy + ly < a.ny;  // and past a ragged end
+            if (!mine) continue;
+            const int at = ly * SW + lx, node = y * a.nx + x;
+            float f[L::Q];
+            if constexpr (FIRST)
+                pull<L, float>(a, x, y, 0, f);
+            else
+                pull_tile<L, PITCH>(a, from, at, x, y, f);
+            if constexpr (LAST)
+                step_body<L, float, CLOSURE, FORMULA, FORCE>(a, f, node);
+            else
+                collide<L, float, CLOSURE, FORMULA, FORCE>(
+                    a, f, node, [&](auto i, float v) { to[CV(i) * PITCH + at] = v; });
+        }
+        if constexpr (!LAST) __syncthreads();
+    });
+}
+
+template <int C, int F, bool FO, int BH>
+cudaError_t launch_block_tile(const StepArgs<float>& a, cudaStream_t s) {
+    auto* k = k_step_block<D2Q9, C, F, FO, BH>;
+    static const cudaError_t ready =
+        cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, block_smem(BH));
+    if (ready != cudaSuccess) return ready;
+    const dim3 grid((a.nx + BW - 1) / BW, (a.ny + BH - 1) / BH);
+    return launch_pdl_smem(k, grid, dim3(BLOCK_THREADS), block_smem(BH), s, a);
+}
+template <int C, int F, bool FO>
+cudaError_t launch_block_form(const StepArgs<float>& a, cudaStream_t s) {
+    const long long tiles = (a.nx + BW - 1LL) / BW * ((a.ny + 19LL) / 20);
+    return tiles >= 152 ? launch_block_tile<C, F, FO, 20>(a, s) : launch_block_tile<C, F, FO, 16>(a, s);
+}
+
+template <int C>
+cudaError_t launch_block_c(const StepArgs<float>& a, int formula, int force, cudaStream_t s) {
+    if (formula == F_YU) return force ? launch_block_form<C, F_YU, true>(a, s) : launch_block_form<C, F_YU, false>(a, s);
+    return force ? launch_block_form<C, F_CHAI, true>(a, s) : launch_block_form<C, F_CHAI, false>(a, s);
+}
+
+}  // namespace lbm

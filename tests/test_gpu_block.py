@@ -1,0 +1,52 @@
+"""Several steps of a small FP32 D2Q9 lattice per launch (shared-memory tiles) against one launch per step: every
+node's arithmetic is the same, so the states are equal bit for bit.  Sizes on and beside the tiles' edges
+(32 x 16, 32 x 20), down to one node; periodic, walled and moving faces; each closure; uniform and field forces;
+step counts that leave a remainder."""
+import numpy as np
+import pytest
+import torch
+
+from test_gpu_parity import Case
+
+pytestmark = pytest.mark.gpu
+
+CAVITY = dict(bc=["wall"] * 3 + ["lid"], lid={3: (0.1, 0.02, 0)})
+CASES = [
+    ((64, 32, 1), "newton", "yu", {}),
+    ((65, 33, 1), "newton", "chai", dict(force=[1e-5, -2e-5])),
+    ((31, 47, 1), "smag", "chai", CAVITY),
+    ((97, 16, 1), "smag", "yu", dict(bc=["periodic"] * 2 + ["wall", "lid"], lid={3: (0.05, 0, 0)}, force=[1e-5, 0])),
+    ((40, 70, 1), "powerlaw", "chai", dict(pl=(0.6, 0.01), **CAVITY)),
+    ((33, 17, 1), "smag_dev", "yu", dict(force_field=True)),
+    ((5, 3, 1), "smag", "yu", dict(force=[1e-5, 0])),
+    ((2, 1, 1), "newton", "yu", {}),
+    ((3, 40, 1), "powerlaw", "yu", dict(pl=(1.3, 0.05), bc=["wall", "lid", "periodic", "periodic"], lid={1: (0, 0.1, 0)})),
+    ((1, 1, 1), "newton", "yu", dict(bc=["wall"] * 4)),
+    ((256, 256, 1), "newton", "yu", CAVITY),
+    ((1283, 83, 1), "smag", "chai", dict(force=[1e-5, 0], **CAVITY)),  # enough tiles for the higher form (32 x 20)
+    ((320, 330, 1), "newton", "yu", {}),
+    ((640, 160, 1), "powerlaw", "chai", dict(pl=(0.6, 0.01), **CAVITY)),
+]
+
+
+@pytest.mark.parametrize("nsteps", [4, 11])
+@pytest.mark.parametrize("dims,closure,formula,extra", CASES)
+def test_blocked_steps_equal_per_step(dims, closure, formula, extra, nsteps):
+    c = Case(9, dims, precision="fp32", closure=closure, formula=formula, tau=0.6, **extra)
+    c.lat.init(c.drho, c.u, c.g)
+    f0 = c.lat.get_state().clone()
+    c.lat.set_schedule("per_step").step(nsteps)
+    ref = c.lat.get_state().clone()
+    c.lat.set_state(f0)
+    before = np.array(c.lat.stats())
+    c.lat.set_schedule("auto").step(nsteps)
+    assert tuple(np.array(c.lat.stats()) - before) == (nsteps, nsteps // 4 + nsteps % 4)
+    got = c.lat.get_state()
+    assert torch.equal(got.view(torch.int32), ref.view(torch.int32)), int((got != ref).sum())
+
+
+def test_lagged_closure_and_large_power_law_lattices_step_one_by_one():
+    for dims, closure in (((64, 32, 1), "smag_lagged"), ((1024, 513, 1), "powerlaw")):
+        c = Case(9, dims, precision="fp32", closure=closure, tau=0.6, pl=(0.7, 0.01))
+        c.lat.init(c.drho, c.u, c.g).step(8)
+        assert c.lat.stats() == (8, 8)
