@@ -57,7 +57,11 @@ cudaError_t launch_step(const StepArgs<typename Store<ST>::R>& a, int closure, i
     const bool yu = formula == F_YU;
     switch (closure) {
         case CL_NEWTON:
-            return launch_step_cf<L, ST, CL_NEWTON, F_YU>(a, force, s);  // either formula (see step_body)
+            // with fixed rates a step needs no S: 16-bit storage steps either formula by the shorter (Yu) moments,
+            // FP32 and FP64 by their own, whose rounding differs (D2Q9 FP32 after 20 steps: Chai's 7.7e-8 from 64
+            // bits, Yu's 9.5e-8)
+            return yu || sizeof(ST) == 2 ? launch_step_cf<L, ST, CL_NEWTON, F_YU>(a, force, s)
+                                         : launch_step_cf<L, ST, CL_NEWTON, sizeof(ST) == 2 ? F_YU : F_CHAI>(a, force, s);
         case CL_SMAG:
             return yu ? launch_step_cf<L, ST, CL_SMAG, F_YU>(a, force, s)
                       : launch_step_cf<L, ST, CL_SMAG, F_CHAI>(a, force, s);

@@ -7,8 +7,7 @@ namespace lbm {
 // margins would each advance, nor for the power law above 2^19 nodes (step_block.cuh).
 cudaError_t block_d2q9_f32(const StepArgs<float>& a, int closure, int formula, int force, cudaStream_t s) {
     switch (closure) {
-        case CL_NEWTON:  // either formula (see collide)
-            return launch_block_c<CL_NEWTON>(a, F_YU, force, s);
+        case CL_NEWTON: return launch_block_c<CL_NEWTON>(a, formula, force, s);
         case CL_SMAG: return launch_block_c<CL_SMAG>(a, formula, force, s);
         case CL_POWERLAW:
             if ((long long)a.nx * a.ny > (1LL << 19)) return cudaErrorNotSupported;

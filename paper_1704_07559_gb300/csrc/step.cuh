@@ -1290,8 +1290,8 @@ __device__ __forceinline__ void strain_split(const StepArgs<RS>& a, const R (&mn
 }
 
 // Everything of a step after the pull, for the node `node`: moments, strain rate by the chosen route,
-// closure, relaxation, force; sink(i, v) takes f*_i.  (With fixed rates a step needs no S, so one kernel,
-// the Yu route's, steps Newtonian lattices of either formula, each viscous moment with its own rate.)
+// closure, relaxation, force; sink(i, v) takes f*_i.  With fixed rates a step needs no S and relaxes each viscous
+// moment at its own rate.
 template <class L, class ST, int CLOSURE, int FORMULA, bool FORCE, class Sink>
 __device__ __forceinline__ void collide(const StepArgs<typename Store<ST>::R>& a, typename Store<ST>::R (&f)[L::Q],
                                         int node, Sink&& sink) {

@@ -310,7 +310,9 @@ cudaError_t launch_stream(const StepArgs<typename Store<ST>::R>& a0, const StepA
     const bool yu = formula == F_YU;
     switch (closure) {
         case CL_NEWTON:
-            return launch_stream_cf<L, ST, CL_NEWTON, F_YU>(a0, a1, c, force, force_stream, s);  // either formula
+            return yu || sizeof(ST) == 2  // as the one-step launch
+                       ? launch_stream_cf<L, ST, CL_NEWTON, F_YU>(a0, a1, c, force, force_stream, s)
+                       : launch_stream_cf<L, ST, CL_NEWTON, sizeof(ST) == 2 ? F_YU : F_CHAI>(a0, a1, c, force, force_stream, s);
         case CL_SMAG:
             return yu ? launch_stream_cf<L, ST, CL_SMAG, F_YU>(a0, a1, c, force, force_stream, s)
                       : launch_stream_cf<L, ST, CL_SMAG, F_CHAI>(a0, a1, c, force, force_stream, s);
@@ -349,9 +351,13 @@ cudaError_t launch_stream(const StepArgs<typename Store<ST>::R>& a0, const StepA
             return force ? launch_stream_ring_form<L, ST, CL_SMAG, F_CHAI, true>(a, c, fs, s)                \
                          : launch_stream_ring_form<L, ST, CL_SMAG, F_CHAI, false>(a, c, fs, s);              \
         }                                                                                                    \
-        if (closure == CL_NEWTON)                                                                            \
-            return force ? launch_stream_ring_form<L, ST, CL_NEWTON, F_YU, true>(a, c, fs, s)                \
-                         : launch_stream_ring_form<L, ST, CL_NEWTON, F_YU, false>(a, c, fs, s);              \
+        if (closure == CL_NEWTON) {                                                                          \
+            if (yu)                                                                                          \
+                return force ? launch_stream_ring_form<L, ST, CL_NEWTON, F_YU, true>(a, c, fs, s)            \
+                             : launch_stream_ring_form<L, ST, CL_NEWTON, F_YU, false>(a, c, fs, s);          \
+            return force ? launch_stream_ring_form<L, ST, CL_NEWTON, F_CHAI, true>(a, c, fs, s)              \
+                         : launch_stream_ring_form<L, ST, CL_NEWTON, F_CHAI, false>(a, c, fs, s);            \
+        }                                                                                                    \
         return cudaErrorNotSupported;                                                                        \
     }                                                                                                        \
     }
