@@ -320,7 +320,9 @@ int lbm_sums_noalloc(int lattice, int nx, int ny, int nz, const lbm_params* p, c
  * Supported: D3Q19, LBM_FP32 or LBM_FP64 populations, LBM_NEWTON or LBM_SMAG, all faces
  * periodic, a force field bound (p->force_field = 1); otherwise LBM_ERR_ARG.
  *  work     caller-owned device workspace of at least lbm_adjoint_workspace() bytes, 256-byte
- *           aligned (checkpoints, segment states, two adjoint buffers, accumulators);
+ *           aligned (checkpoints, segment states, two adjoint buffers, accumulators).  With at
+ *           least lbm_adjoint_workspace(T, T) bytes every state is kept and none recomputed (T
+ *           forward steps in all); the results are the same bit for bit;
  *  dLdg     device pointer to 3 x N doubles, overwritten with dL/dg (component-major);
  *  loss     HOST pointer to one double, set to L.
  * After the call the current buffer holds the state after T steps.  Synchronises the stream. */

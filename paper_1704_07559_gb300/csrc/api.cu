@@ -548,7 +548,8 @@ AdjLayout adjoint_layout(const lbm_ctx* c, int T, int seg) {
 }
 
 template <class R>
-cudaError_t adjoint_run(lbm_ctx* c, int T, int seg, char* work, const AdjLayout& L, double* dLdg, double* loss) {
+cudaError_t adjoint_run(lbm_ctx* c, int T, int seg, bool keep_all, char* work, const AdjLayout& L, double* dLdg,
+                        double* loss) {
     cudaStream_t s = c->stream;
     cudaError_t e;
     const size_t state_bytes = (size_t)c->q * c->stride * c->elem_bytes;
@@ -568,36 +569,31 @@ cudaError_t adjoint_run(lbm_ctx* c, int T, int seg, char* work, const AdjLayout&
 
     const long long ring = (long long)(L.state / c->elem_bytes);  // elements between segment states
     const int forced = c->schedule == LBM_SCHEDULE_STREAM ? 1 : 0;
-    // states 1 .. m - 1 of segment sgi into the segment buffers sg(0 .. m - 2), from its checkpoint:
-    // the first step from the checkpoint, the rest (FP32, where the schedule allows) in one ring
-    // launch that writes each step to the next state buffer
-    auto fill_segment = [&](int sgi, int m) -> cudaError_t {
+    // n steps from the state `first`, each written to the next of the equally spaced state buffers after it:
+    // in one ring launch (FP32, where the schedule allows) or step by step
+    auto run_along = [&](char* first, int n) -> cudaError_t {
         cudaError_t err;
-        int i = 1;
-        if (m >= 2) {
-            err = run_step(c, cp(sgi), sg(0));
-            if (err != cudaSuccess) return err;
-            i = 2;
-        }
         if constexpr (!F64) {
-            if (m - 2 >= 2 && c->schedule != LBM_SCHEDULE_PER_STEP) {
+            if (n >= 2 && c->schedule != LBM_SCHEDULE_PER_STEP) {
                 lbm::StepArgs<float> ra;
                 fill_args(c, &ra);
-                ra.S_out = ra.tau_out = ra.drho_out = ra.u_out = nullptr;
-                set_buffers(c, &ra, sg(0), sg(1));
-                const lbm::StreamCtl ctl = {c->sync, m - 2, c->stream_rows, c->stream_tiles, 0, ring};
+                set_buffers(c, &ra, first, first + L.state);
+                const lbm::StreamCtl ctl = {c->sync, n, c->stream_rows, c->stream_tiles, 0, ring};
                 err = lbm::stream_ring_d3q19_f32(ra, ctl, c->p.closure, c->p.formula, has_force(c) ? 1 : 0, forced, s);
-                if (err == cudaSuccess)
-                    i = m;
-                else if (err != cudaErrorNotSupported)
-                    return err;
+                if (err != cudaErrorNotSupported) return err;
             }
         }
-        for (; i < m; ++i) {
-            err = run_step(c, sg(i - 2), sg(i - 1));
+        for (int i = 0; i < n; ++i) {
+            err = run_step(c, first + i * L.state, first + (i + 1) * L.state);
             if (err != cudaSuccess) return err;
         }
         return cudaSuccess;
+    };
+    // states 1 .. m - 1 of segment sgi into the segment buffers sg(0 .. m - 2), from its checkpoint
+    auto fill_segment = [&](int sgi, int m) -> cudaError_t {
+        if (m < 2) return cudaSuccess;
+        cudaError_t err = run_step(c, cp(sgi), sg(0));
+        return err == cudaSuccess ? run_along(static_cast<char*>(sg(0)), m - 2) : err;
     };
 
     // forward T steps from the current state, keeping every seg-th state: per segment, the first
@@ -606,12 +602,21 @@ cudaError_t adjoint_run(lbm_ctx* c, int T, int seg, char* work, const AdjLayout&
     // next checkpoint.  The last segment writes its states straight into the segment buffers the
     // reverse sweep reads (so it needs no recomputation there) and its last step the final state
     // into a context buffer.
+    // With room for every state (keep_all) the sweep writes state k to work + k L.state instead, and the
+    // reverse sweep recomputes nothing.
     const void* fcur = c->buf[c->cur];
     bool last_filled = false;
     if (T > 0) {
         e = cudaMemcpyAsync(cp(0), c->buf[c->cur], state_bytes, cudaMemcpyDeviceToDevice, s);
         if (e != cudaSuccess) return e;
-        for (int k0 = 0; k0 < T; k0 += seg) {
+        if (keep_all) {
+            e = run_along(work, T - 1);
+            if (e != cudaSuccess) return e;
+            e = run_step(c, work + (size_t)(T - 1) * L.state, c->buf[0]);
+            if (e != cudaSuccess) return e;
+            c->cur = 0;
+        }
+        for (int k0 = 0; k0 < T && !keep_all; k0 += seg) {
             const int k1 = (k0 + seg < T) ? k0 + seg : T;
             const bool to_cp = k1 < T;
             if (to_cp && k1 - k0 == 1) {  // one-step segments: checkpoint to checkpoint
@@ -664,31 +669,33 @@ cudaError_t adjoint_run(lbm_ctx* c, int T, int seg, char* work, const AdjLayout&
     // reverse sweep, segment by segment from the last, recomputing the states of every segment but
     // the last
     int lc = 0;
-    for (int sgi = L.ncp - 1; sgi >= 0; --sgi) {
+    const int nsegs = T > 0 ? (T + seg - 1) / seg : 0;
+    for (int sgi = nsegs - 1; sgi >= 0; --sgi) {
         const int k0 = sgi * seg, k1 = (k0 + seg < T) ? k0 + seg : T, m = k1 - k0;
         const void* states[1024];
-        states[0] = cp(sgi);
-        for (int i = 1; i < m; ++i) states[i] = sg(i - 1);
+        for (int i = 0; i < m; ++i)
+            states[i] = keep_all ? work + (size_t)(k0 + i) * L.state : (i == 0 ? cp(sgi) : sg(i - 1));
         // recompute the segment's states (the last segment's are still there from the forward sweep)
-        if (!(sgi == L.ncp - 1 && last_filled)) {
+        if (!keep_all && !(sgi == nsegs - 1 && last_filled)) {
             e = fill_segment(sgi, m);
             if (e != cudaSuccess) return e;
         }
-        // reverse steps k1 - 1 .. k0 + 1 (states sg(m - 2) down to sg(0), equally spaced) in one
-        // launch where the schedule allows, the rest one launch per step
+        // reverse steps k1 - 1 .. k0 + 1 (states sg(m - 2) down to sg(0), equally spaced; with every state kept
+        // also k0) in one launch where the schedule allows, the rest one launch per step
         int n = k1 - 1;
         if constexpr (!F64) {
-            if (m - 1 >= 2 && c->schedule != LBM_SCHEDULE_PER_STEP) {
+            const int spaced = keep_all ? m : m - 1;
+            if (spaced >= 2 && c->schedule != LBM_SCHEDULE_PER_STEP) {
                 lbm::AdjArgs<R> b0 = a, b1 = a;
                 set_buffers(c, &b0.st, states[m - 1], nullptr);
                 set_buffers(c, &b1.st, states[m - 1], nullptr);
                 lbm::set_lambda(&b0, static_cast<const R*>(lam[lc]), lam[1 - lc]);
                 lbm::set_lambda(&b1, static_cast<const R*>(lam[1 - lc]), lam[lc]);
-                const lbm::StreamCtl ctl = {c->sync, m - 1, c->stream_rows, c->stream_tiles, 0, ring};
+                const lbm::StreamCtl ctl = {c->sync, spaced, c->stream_rows, c->stream_tiles, 0, ring};
                 e = lbm::adj_stream_f32(b0, b1, ctl, c->p.closure, forced, s);
                 if (e == cudaSuccess) {
-                    n = k0;
-                    if ((m - 1) & 1) lc = 1 - lc;
+                    n = k1 - 1 - spaced;
+                    if (spaced & 1) lc = 1 - lc;
                 } else if (e != cudaErrorNotSupported) {
                     return e;
                 }
@@ -707,7 +714,7 @@ cudaError_t adjoint_run(lbm_ctx* c, int T, int seg, char* work, const AdjLayout&
         e = fold(dF);
         if (e != cudaSuccess) return e;
     }
-    if (L.ncp == 0) {  // T = 0: only the functional's direct term
+    if (nsegs == 0) {  // T = 0: only the functional's direct term
         e = fold(dF);
         if (e != cudaSuccess) return e;
     }
@@ -1166,11 +1173,15 @@ int lbm_adjoint(lbm_ctx* c, int T, int seg, void* work, int64_t work_bytes, doub
     if (seg > 1024) return fail(c, LBM_ERR_ARG, "lbm_adjoint: seg <= 1024");
     if (!work || !dLdg || !loss) return fail(c, LBM_ERR_ARG, "lbm_adjoint: work, dLdg and loss are required");
     if ((uintptr_t)work & 255) return fail(c, LBM_ERR_ARG, "lbm_adjoint: workspace must be 256-byte aligned");
-    const AdjLayout L = adjoint_layout(c, T, seg);
+    AdjLayout L = adjoint_layout(c, T, seg);
     if (work_bytes < (int64_t)L.total) return fail(c, LBM_ERR_ARG, "lbm_adjoint: workspace too small");
+    // room for every state: keep them all (the layout of one segment of T steps)
+    const AdjLayout all = adjoint_layout(c, T, T > 0 ? T : 1);
+    const bool keep_all = T > 0 && work_bytes >= (int64_t)all.total;
+    if (keep_all) L = all;
     cudaError_t e = c->p.precision == LBM_FP64
-                        ? adjoint_run<double>(c, T, seg, static_cast<char*>(work), L, dLdg, loss)
-                        : adjoint_run<float>(c, T, seg, static_cast<char*>(work), L, dLdg, loss);
+                        ? adjoint_run<double>(c, T, seg, keep_all, static_cast<char*>(work), L, dLdg, loss)
+                        : adjoint_run<float>(c, T, seg, keep_all, static_cast<char*>(work), L, dLdg, loss);
     if (e != cudaSuccess) return cuda_fail(c, e, "lbm_adjoint");
     c->watch_ref_ok = 0;  // the current state is now the one after T steps
     if (!is_finite(*loss)) return fail(c, LBM_ERR_NONFINITE, "lbm_adjoint: non-finite functional");
