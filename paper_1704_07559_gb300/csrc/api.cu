@@ -650,6 +650,8 @@ cudaError_t adjoint_run(lbm_ctx* c, int T, int seg, bool keep_all, char* work, c
     lbm::AdjArgs<R> a;
     fill_args(c, &a.st);
     a.dF = dF;
+    a.acc_read = 1;
+    a.fold = nullptr;
     a.partial = partial;
     // the functional at f^T: loss partials, lambda_T, dF
     set_buffers(c, &a.st, fcur, nullptr);
@@ -667,7 +669,8 @@ cudaError_t adjoint_run(lbm_ctx* c, int T, int seg, bool keep_all, char* work, c
     if (e != cudaSuccess) return e;
 
     // reverse sweep, segment by segment from the last, recomputing the states of every segment but
-    // the last
+    // the last.  A segment's gradient starts from zero (the last one's from the functional's direct term) and its last
+    // step adds it to dLdg in FP64.
     int lc = 0;
     const int nsegs = T > 0 ? (T + seg - 1) / seg : 0;
     for (int sgi = nsegs - 1; sgi >= 0; --sgi) {
@@ -687,6 +690,8 @@ cudaError_t adjoint_run(lbm_ctx* c, int T, int seg, bool keep_all, char* work, c
             const int spaced = keep_all ? m : m - 1;
             if (spaced >= 2 && c->schedule != LBM_SCHEDULE_PER_STEP) {
                 lbm::AdjArgs<R> b0 = a, b1 = a;
+                b0.acc_read = b1.acc_read = sgi == nsegs - 1;
+                b0.fold = b1.fold = spaced == m ? dLdg : nullptr;
                 set_buffers(c, &b0.st, states[m - 1], nullptr);
                 set_buffers(c, &b1.st, states[m - 1], nullptr);
                 lbm::set_lambda(&b0, static_cast<const R*>(lam[lc]), lam[1 - lc]);
@@ -704,6 +709,8 @@ cudaError_t adjoint_run(lbm_ctx* c, int T, int seg, bool keep_all, char* work, c
         for (; n >= k0; --n) {
             set_buffers(c, &a.st, states[n - k0], nullptr);
             lbm::set_lambda(&a, static_cast<const R*>(lam[lc]), lam[1 - lc]);
+            a.acc_read = n < k1 - 1 || sgi == nsegs - 1;
+            a.fold = n == k0 ? dLdg : nullptr;
             if constexpr (F64)
                 e = lbm::adj_step_f64(a, c->p.closure, s);
             else
@@ -711,8 +718,6 @@ cudaError_t adjoint_run(lbm_ctx* c, int T, int seg, bool keep_all, char* work, c
             if (e != cudaSuccess) return e;
             lc = 1 - lc;
         }
-        e = fold(dF);
-        if (e != cudaSuccess) return e;
     }
     if (nsegs == 0) {  // T = 0: only the functional's direct term
         e = fold(dF);

@@ -277,8 +277,8 @@ class Lattice:
 
     def adjoint(self, T, seg=None):
         """(L, dL/dg) after T steps from the current state: L as a float, dL/dg as a float64
-        tensor (d, nz, ny, nx).  seg defaults to round(sqrt(T)); then, where T states take at most a
-        quarter of the memory free on the device, all of them are kept instead of recomputing
+        tensor (d, nz, ny, nx).  seg defaults to round(sqrt(T)); then, where T states take at most an
+        eighth of the device's memory and that much is free, all of them are kept instead of recomputing
         each segment (the same result, T forward steps instead of about 2T).  A given seg bounds the
         memory as lbm_adjoint_workspace states it.  The current state afterwards is the state after
         T steps."""
@@ -291,13 +291,12 @@ class Lattice:
         if not given and 1 < T <= 1024:
             every = ctypes.c_int64()
             self._check(L.lbm_adjoint_workspace(self.ctx, T, T, ctypes.byref(every)))
-            cached = torch.cuda.memory_reserved(self.device) - torch.cuda.memory_allocated(self.device)
-            if every.value <= (torch.cuda.mem_get_info(self.device)[0] + cached) // 4:
+            if every.value <= torch.cuda.get_device_properties(self.device).total_memory // 8:
                 try:
                     work = torch.empty(every.value + 256, dtype=torch.uint8, device=self.device)
                     nbytes = every
                 except torch.cuda.OutOfMemoryError:
-                    work = None
+                    pass
         if work is None:
             work = torch.empty(nbytes.value + 256, dtype=torch.uint8, device=self.device)
         off = (-work.data_ptr()) % 256

@@ -42,7 +42,16 @@ def test_without_room_the_checkpoints_are_used(monkeypatch):
     lat.init(np.zeros((8, 8, 16)), 0.01 * np.ones((3, 8, 8, 16)))
     f0 = lat.get_state().clone()
     a = lat.adjoint(9)
-    monkeypatch.setattr(torch.cuda, "mem_get_info", lambda *_: (0, 0))
+    sizes, empty = [], torch.empty
+
+    def scarce(*shape, **kw):  # the first allocation, room for every state, fails
+        sizes.append(shape[0])
+        if len(sizes) == 1:
+            raise torch.cuda.OutOfMemoryError("out of memory")
+        return empty(*shape, **kw)
+
     lat.set_state(f0)
+    monkeypatch.setattr(torch, "empty", scarce)
     b = lat.adjoint(9)
+    assert sizes[1] < sizes[0]
     assert a[0] == b[0] and torch.equal(a[1], b[1])
