@@ -18,6 +18,8 @@
 // 70.2 / 63.5 / 67.2 and 4096^2 84 / 72 / 77, so it takes this form up to 2^19 nodes only.
 #pragma once
 
+#include <atomic>
+
 #include "launch.h"
 #include "step.cuh"
 
@@ -109,9 +111,16 @@ __global__ void __launch_bounds__(BLOCK_THREADS) k_step_block(const StepArgs<flo
 template <int C, int F, bool FO, int BH>
 cudaError_t launch_block_tile(const StepArgs<float>& a, cudaStream_t s) {
     auto* k = k_step_block<D2Q9, C, F, FO, BH>;
-    static const cudaError_t ready =
-        cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, block_smem(BH));
-    if (ready != cudaSuccess) return ready;
+    // the kernel's shared-memory limit is set once per device
+    static std::atomic<unsigned long long> ready{0};
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    if (dev >= 64 || !((ready.load() >> dev) & 1)) {
+        e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, block_smem(BH));
+        if (e != cudaSuccess) return e;
+        if (dev < 64) ready.fetch_or(1ull << dev);
+    }
     const dim3 grid((a.nx + BW - 1) / BW, (a.ny + BH - 1) / BH);
     return launch_pdl_smem(k, grid, dim3(BLOCK_THREADS), block_smem(BH), s, a);
 }

@@ -218,17 +218,19 @@ int resident_blocks(K kernel) {
     return (per_sm < 1 ? 1 : per_sm) * sms;
 }
 
-// Unit height: c.rows (about 1024 nodes) times the largest m in {4, 2, 1} that still leaves more
-// units than resident blocks plus the span of positions a unit's dependencies reach ahead of it
-// (two planes of bands and two bands; no planes when nz = 1), so that no block waits; false when
-// even m = 1 does not.
+// Unit height: c.rows (about 1024 nodes) times the largest m in {4, 2, 1} that still leaves a quarter more
+// units than resident blocks, beyond the span of positions a unit's dependencies reach ahead of it (two
+// planes of bands and two bands; no planes when nz = 1), so that blocks seldom wait; false when even m = 1
+// does not.  (With no more than the resident blocks and the span: 112^3, 1456 units for 1368 + 29, 38.2 GLUPS
+// against 40.9 one launch per step; FP16 104^3, 1248 for 1064 + 27, 60.9 against 66.6; 120^3, 1800 for 1368 + 33,
+// 43.2 against 41.6.)
 inline bool pick_units(const StreamCtl& base, int ny, int nz, int resident, StreamCtl* out) {
     for (int m = 4; m >= 1; m /= 2) {
         const int rows = base.rows * m < ny ? base.rows * m : ny;
         const int tiles = (ny + rows - 1) / rows;
         const long long units = (long long)nz * tiles;
         const long long span = (nz > 1 ? 2LL * tiles : 0) + 3;
-        if (units >= resident + span) {
+        if (units >= resident + resident / 4 + span) {
             *out = base;
             out->rows = rows;
             out->tiles_y = tiles;
@@ -250,6 +252,10 @@ cudaError_t launch_stream_form(const StepArgs<typename Store<ST>::R>& a0, const 
                                const StreamCtl& c, bool force_stream, cudaStream_t s) {
     const long long N = (long long)a0.nx * a0.ny * a0.nz;
     if (!force_stream && N > (1LL << 23)) return cudaErrorNotSupported;
+    // FP32 rows that do not start on a 32-byte boundary: one launch per step is the faster (GLUPS, streamed / per
+    // step: 97x150x97 35.5 / 37.9, 121 37.2 / 38.9, 150 38.9 / 39.8, 250 40.1 / 41.4; but 160 42.8 / 40.2, 200 41.2 /
+    // 41.0, 224 43.0 / 41.3)
+    if (!force_stream && sizeof(ST) == 4 && a0.nx % 8 != 0) return cudaErrorNotSupported;
     StreamCtl u;
     if constexpr (sizeof(ST) == 2) {
         if (a0.nx % 2 == 0) {
