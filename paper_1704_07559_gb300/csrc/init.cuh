@@ -10,7 +10,7 @@
 //
 // What bounds it: 180 B a node with a gradient (FP32), and the arithmetic.  In FP64 the population-
 // by-population form took about 530 FP64 operations a node on the pipe that finishes 2 a clock and SM:
-// 5.9 ms for a 192^3 FP32 box with a gradient, now 0.69 ms (its bytes take 0.19 ms at the measured copy
+// 5.9 ms for a 192^3 FP32 box with a gradient, now 0.35 ms (its bytes take 0.19 ms at the measured copy
 // bandwidth; the error against 64 bits is unchanged, 2.5e-8).  FP64 storage runs the pair form above in FP64; the other storages run it in
 // pairs of floats (dfloat.cuh: 48 bits, rounded once to FP32 at the end, as the FP64 result was), and
 // only nodes next to a moving wall or with a result that is not finite repeat it in FP64.
@@ -240,23 +240,31 @@ __device__ __forceinline__ bool init_at(const StepArgs<double>& a, const InitCon
                                         const typename Store<ST>::R* __restrict__ ffield,
                                         V (&f)[L::Q], V& tau_out) {
     const long long N = (long long)a.nx * a.ny * a.nz;  // component offsets (up to 8N) exceed 2^31 on big grids
+    // every load first: the conversions branch, and a load behind a branch waits for it (192^3, with the blocks
+    // cut at row ends that left a quarter of the threads idle: 0.60 ms)
+    double du[3] = {0.0, 0.0, 0.0}, dg[9];
+    typename Store<ST>::R dF[3];
+    const double dd = drho[node];
+    sfor<L::D>([&](auto d) { du[d] = u[CV(d) * N + node]; });
+    if (gu) sfor<L::D * L::D>([&](auto c) { dg[c] = gu[CV(c) * N + node]; });
+    if constexpr (FORCE) {
+        if (ffield) sfor<L::D>([&](auto d) { dF[d] = ffield[CV(d) * N + node]; });
+    }
     X j[3], F[3], G[3][3];
     sfor<3>([&](auto d) {
         F[d] = k.F[CV(d)];
         sfor<3>([&](auto e) { G[CV(d)][CV(e)] = X(0.0f); });
     });
     sfor<L::D>([&](auto d) {
-        j[d] = k.r0 * XC<X>::in(u[CV(d) * N + node]);
+        j[d] = k.r0 * XC<X>::in(du[d]);
         if constexpr (FORCE) {
-            if (ffield) F[d] = XC<X>::in(ffield[CV(d) * N + node]);
+            if (ffield) F[d] = XC<X>::in(dF[d]);
         }
     });
-    const X dr = XC<X>::in(drho[node]);
+    const X dr = XC<X>::in(dd);
     if (gu)
         sfor<L::D>([&](auto p) {
-            sfor<L::D>([&](auto q) {
-                G[CV(p)][CV(q)] = k.r0 * XC<X>::in(gu[(CV(p) * L::D + CV(q)) * N + node]);
-            });
+            sfor<L::D>([&](auto q) { G[CV(p)][CV(q)] = k.r0 * XC<X>::in(dg[CV(p) * L::D + CV(q)]); });
         });
     const X tau = init_tau<L>(a, k, G);
     tau_out = XC<X>::template out<V>(tau);
@@ -282,15 +290,14 @@ __device__ __noinline__ void init_again(const StepArgs<double>& a, const InitCon
 
 template <class L, class ST, bool FORCE>
 __global__ void __launch_bounds__(128) k_init(const StepArgs<double> a, const InitConst<InitX<ST>> k,
-                                              const InitConst<double> kd, const double* __restrict__ drho,
+                                              const InitConst<double> kd, const NodeMap g,
+                                              const double* __restrict__ drho,
                                               const double* __restrict__ u, const double* __restrict__ gu,
                                               const typename Store<ST>::R* __restrict__ ffield,
                                               typename Store<ST>::R* __restrict__ tau_field) {
     using R = typename Store<ST>::R;
-    const int x = blockIdx.x * blockDim.x + threadIdx.x;
-    const int y = blockIdx.y * blockDim.y + threadIdx.y;
-    const int z = blockIdx.z + a.z0;
-    if (x >= a.nx || y >= a.ny) return;
+    int x, y, z;
+    if (!node_in_order<1>(a, g, x, y, z)) return;
     const int node = (z * a.ny + y) * a.nx + x;
     R f[L::Q], tau;
     bool ok = init_at<L, ST, FORCE>(a, k, node, drho, u, gu, ffield, f, tau);

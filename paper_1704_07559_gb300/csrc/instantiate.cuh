@@ -88,14 +88,15 @@ cudaError_t launch_step(const StepArgs<typename Store<ST>::R>& a, int closure, i
 template <class L, class ST>
 cudaError_t launch_init(const StepArgs<double>& a, int closure, const double* drho, const double* u, const double* gu,
                         const typename Store<ST>::R* ffield, typename Store<ST>::R* tau_field, cudaStream_t s) {
-    dim3 g, b;
-    lattice_grid(a.nx, a.ny, a.nzc, &g, &b);
+    constexpr int b = sizeof(ST) == 8 ? 64 : 128;
+    const NodeMap m = node_map<1>(a);
+    const dim3 g((unsigned)((m.threads + (long long)b - 1) / b));
     const InitConst<InitX<ST>> k = init_const<L, InitX<ST>>(a, closure);
     const InitConst<double> kd = init_const<L, double>(a, closure);
     if (ffield || a.F[0] != 0.0 || a.F[1] != 0.0 || a.F[2] != 0.0)
-        k_init<L, ST, true><<<g, b, 0, s>>>(a, k, kd, drho, u, gu, ffield, tau_field);
+        k_init<L, ST, true><<<g, b, 0, s>>>(a, k, kd, m, drho, u, gu, ffield, tau_field);
     else
-        k_init<L, ST, false><<<g, b, 0, s>>>(a, k, kd, drho, u, gu, ffield, tau_field);
+        k_init<L, ST, false><<<g, b, 0, s>>>(a, k, kd, m, drho, u, gu, ffield, tau_field);
     return cudaGetLastError();
 }
 

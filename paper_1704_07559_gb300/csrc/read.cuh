@@ -64,7 +64,9 @@ __global__ void __launch_bounds__(128) k_macro(const StepArgs<typename Store<ST>
 // with an error-free two-sum (hi, lo) pair per component, FP64 states in plain FP64; per-block
 // partials go to scratch as FP64 and one ordered pass adds them.  A thread waits for one node's
 // populations at a time, so with FP32 arithmetic it fetches its next node's before adding the first's
-// (the order of the additions is the same): 200x150x97 FP32 channel 72 -> 57 us (its bytes: 33 us).
+// (the order of the additions is the same): 200x150x97 FP32 channel 72 -> 57 us (its bytes: 33 us), and with
+// every block resident (80 registers left the fourth of each SM to a second round) the three read-outs of a pass
+// 199 -> 178 us.
 
 constexpr int SUM_THREADS = 256;
 
@@ -99,8 +101,9 @@ __device__ __forceinline__ void sum_node(const StepArgs<R>& a, const R (&f)[L::Q
         acc[1 + d].add(fma(R(0.5), a.force_field ? a.force_field[d * N + n] : a.F[d], mj[d]));
 }
 
+// FP32 is held to 64 registers, so that the grid's four blocks per SM are resident together.
 template <class L, class ST>
-__global__ void __launch_bounds__(SUM_THREADS) k_sums(const StepArgs<typename Store<ST>::R> a, double* __restrict__ partial) {
+__global__ void __launch_bounds__(SUM_THREADS, sizeof(typename Store<ST>::R) == 4 ? SUM_BLOCKS / 152 : 0) k_sums(const StepArgs<typename Store<ST>::R> a, double* __restrict__ partial) {
     using R = typename Store<ST>::R;
     constexpr int D = L::D;
     constexpr bool AHEAD = sizeof(R) == 4;
