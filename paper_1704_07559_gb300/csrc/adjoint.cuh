@@ -15,9 +15,6 @@
 // sigma = S' + tau' 3Cs^2 (2 w S/|S|)/(1 + 3Cs^2 s^2 2 (w S).B/|S|); TF' = -D'/|T|^2 + mn'/2;
 // m_eq' = -mn'; drho' = -11 m_eq'_1 + 3 m_eq'_2; j' = J^T m_eq' + sum_k TF'_k H_k F (H_k the
 // constant Hessian of m_eq_k in j); F' = J^T TF' + j'/2; p' = lambda + T^T (drho', ..., j', mn').
-// With q_k = (T lambda)_k / |T_k|^2 (so TF' = q + mn'/2) the halves of J^T mn' in F' cancel:
-// F' = (H F)/2 + J^T q, H = sum_k TF'_k H_k; and J's j-dependent rows and H are symmetric 3x3 forms of mn'
-// and q (sym_form).
 // Both strain routes compute the same function (Sec. 5.1), so one derivative serves both.
 //
 // Adjoint streaming: p_i(x) = f_i(x - c_i), so lambda_n,i(y) = mu_i(y + c_i) where mu = p' of
@@ -40,36 +37,29 @@ struct NodeFwd {
 
 template <class R>
 __device__ __forceinline__ R strain_w_dot(const R (&S)[6], const R (&T)[6]) {
-    return fma(S[0], T[0], fma(S[1], T[1], S[2] * T[2])) + R(2) * fma(S[3], T[3], fma(S[4], T[4], S[5] * T[5]));
+    return S[0] * T[0] + S[1] * T[1] + S[2] * T[2] + R(2) * (S[3] * T[3] + S[4] * T[4] + S[5] * T[5]);
 }
 
-// M(v), the symmetric form with sum_k v_k H_k a = M(v) a / rho0 for any vector a (H_k: the Hessian of m_eq_k in j;
-// xx, yy, zz, xy, yz, xz), so that J(j)^T v = M(v) j / rho0 + (v_3 - 2/3 v_4, v_5 - 2/3 v_6, v_7 - 2/3 v_8)
+// J(jv)^T v for the 19-vector v (only entries 1..15 enter), J = d m_eq / d j at j = jv
 template <class R>
-__device__ __forceinline__ void sym_form(const R (&v)[19], R (&M)[6]) {
-    const R e = fma(R(38.0f), v[1], R(-11.0f) * v[2]);
-    const R a9 = fma(R(-0.5f), v[10], v[9]), a11 = fma(R(-0.5f), v[12], v[11]);
-    const R f = fma(R(-2.0f), a9, e);
-    M[0] = fma(R(4.0f), a9, e);
-    M[1] = fma(R(2.0f), a11, f);
-    M[2] = fma(R(-2.0f), a11, f);
-    M[3] = v[13];
-    M[4] = v[14];
-    M[5] = v[15];
-}
-// out = M a + b
-template <class R>
-__device__ __forceinline__ void sym_apply(const R (&M)[6], const R (&a)[3], const R (&b)[3], R (&out)[3]) {
-    out[0] = fma(M[0], a[0], fma(M[3], a[1], fma(M[5], a[2], b[0])));
-    out[1] = fma(M[3], a[0], fma(M[1], a[1], fma(M[4], a[2], b[1])));
-    out[2] = fma(M[5], a[0], fma(M[4], a[1], fma(M[2], a[2], b[2])));
+__device__ __forceinline__ void jt(const R (&jv)[3], const R (&v)[19], R ir0, R (&out)[3]) {
+    const R a9 = v[9] - R(0.5) * v[10], a11 = v[11] - R(0.5) * v[12];
+    const R e = R(38) * v[1] - R(11) * v[2];
+    out[0] = ir0 * (e * jv[0] + R(4) * jv[0] * a9 + jv[1] * v[13] + jv[2] * v[15]) + v[3] - cst<R>(2.0 / 3.0) * v[4];
+    out[1] = ir0 * (e * jv[1] - R(2) * jv[1] * a9 + R(2) * jv[1] * a11 + jv[0] * v[13] + jv[2] * v[14]) + v[5] -
+             cst<R>(2.0 / 3.0) * v[6];
+    out[2] = ir0 * (e * jv[2] - R(2) * jv[2] * a9 - R(2) * jv[2] * a11 + jv[1] * v[14] + jv[0] * v[15]) + v[7] -
+             cst<R>(2.0 / 3.0) * v[8];
 }
 
 // forward map of one node (Yu form, Smagorinsky or Newtonian closure)
 template <int CLOSURE, class R>
 __device__ __forceinline__ void node_forward(const R (&p)[19], const R (&F)[3], const StepArgs<R>& a, NodeFwd<R>& st) {
     R P[9], Dd[9], m[19];
-    pair_sums<D3Q19>(p, P, Dd);
+    sfor<9>([&](auto q) {
+        P[q] = p[D3Q19::pa(CV(q))] + p[D3Q19::pb(CV(q))];
+        Dd[q] = p[D3Q19::pa(CV(q))] - p[D3Q19::pb(CV(q))];
+    });
     Xf<D3Q19>::forward(p[0], P, Dd, m);
     const R ir0 = a.inv_rho0;
     R u[3], meq[19], TF[19];
@@ -91,98 +81,100 @@ __device__ __forceinline__ void node_forward(const R (&p)[19], const R (&F)[3], 
     R A[6];
     Eq<D3Q19>::yu_split(st.mn, a.s[1] * R(Eq<D3Q19>::YU_A) * ir0, ir0, A, st.B);
     st.tau = solve_tau<D3Q19, R, CLOSURE, false>(A, st.B, a, st.S, st.s, 0);  // Newtonian / Smagorinsky only
-    st.snorm = c_sqrt(R(2) * strain_w_dot(st.S, st.S));
+    st.snorm = sqrt(R(2) * strain_w_dot(st.S, st.S));
 }
 
-// Reverse map of one node.  lam: adjoint of f* (HAS_LAM, a reverse step), or Sbar, taubar_d: direct adjoints of
-// S and tau (the functional).  Outputs mu = dL/dp and Fbar = dL/dF at the node.
+// Reverse map of one node.  lam: adjoint of f* (ignored when HAS_LAM is false); Sbar, taubar_d:
+// direct adjoints of S and tau.  Outputs mu = dL/dp and Fbar = dL/dF at the node.
 template <int CLOSURE, bool HAS_LAM, class R>
 __device__ __forceinline__ void node_backward(const NodeFwd<R>& st, const R (&lam)[19], const R (&Sbar)[6], R taubar_d,
                                               const StepArgs<R>& a, R (&mu)[19], R (&Fbar)[3]) {
     const R ir0 = a.inv_rho0;
-    R q[19];  // (T lam)_k / |T_k|^2
+    R Db[19];  // D' = -T lam
     if constexpr (HAS_LAM) {
-        R P[9], Dd[9];
-        pair_sums<D3Q19>(lam, P, Dd);
-        Xf<D3Q19>::forward(lam[0], P, Dd, q);
-        sfor<19>([&](auto k) { q[k] = cst<R>(1.0 / norm2<D3Q19>(CV(k))) * q[k]; });
-    }
-    // sigma, the adjoint of S with tau's share
-    R sig[6];
-    sfor<6>([&](auto c) { sig[c] = HAS_LAM ? R(0.0f) : Sbar[c]; });
-    if constexpr (CLOSURE != CL_NEWTON) {
-        // tau' = (direct) - s' s^2, s' = S'.B - sum_visc q_k mn_k
-        R taubar;
-        if constexpr (HAS_LAM) {
-            R sum = R(0.0f);
-            sfor<19>([&](auto k) {
-                if constexpr (D3Q19::viscous(CV(k))) sum = fma(q[k], st.mn[k], sum);
-            });
-            taubar = sum * (st.s * st.s);
-        } else {
-            R sbar = R(0.0f);
-            sfor<6>([&](auto c) { sbar = fma(Sbar[c], st.B[c], sbar); });
-            taubar = fma(-sbar, st.s * st.s, taubar_d);
-        }
-        if (st.snorm > R(0)) {
-            const R c3 = R(2.0f) * a.smag_c3;
-            const R den = fma(c3 * (st.s * st.s), strain_w_dot(st.S, st.B), st.snorm);
-            const R coef = taubar * c3 * c_rcp(den);
-            sfor<6>([&](auto c) {
-                const R w = CV(c) < 3 ? coef : R(2.0f) * coef;
-                sig[c] = HAS_LAM ? w * st.S[c] : fma(w, st.S[c], sig[c]);
-            });
-        }
-    }
-    // mn' = Y^T(sigma) - s_k q_k
-    R mnb[19];
-    sfor<19>([&](auto k) { mnb[k] = R(0.0f); });
-    if constexpr (CLOSURE != CL_NEWTON || !HAS_LAM) {
-        const R si = st.s * ir0, s12 = sig[1] + sig[2];
-        mnb[1] = -(a.s[1] * R(Eq<D3Q19>::YU_A) * ir0) * (sig[0] + s12);
-        mnb[9] = si * fma(R(0.25f), s12, R(-0.5f) * sig[0]);
-        mnb[11] = (R(0.75f) * si) * (sig[2] - sig[1]);
-        mnb[13] = (R(-1.5f) * si) * sig[3];
-        mnb[14] = (R(-1.5f) * si) * sig[4];
-        mnb[15] = (R(-1.5f) * si) * sig[5];
-    }
-    if constexpr (HAS_LAM)
-        sfor<19>([&](auto k) {
-            if constexpr (!D3Q19::conserved(CV(k)))
-                mnb[k] = fma(D3Q19::viscous(CV(k)) ? -st.s : -a.s[k], q[k], mnb[k]);
+        R P[9], Dd[9], Lm[19];
+        sfor<9>([&](auto q) {
+            P[q] = lam[D3Q19::pa(CV(q))] + lam[D3Q19::pb(CV(q))];
+            Dd[q] = lam[D3Q19::pa(CV(q))] - lam[D3Q19::pb(CV(q))];
         });
-    // j' = H F - J^T mn', F' = (H F)/2 + J^T q with H = M(mn'/2 + q)/rho0
-    R A[6], j[3], F[3], hF[3], Aj[3];
-    for (int d = 0; d < 3; ++d) {
-        j[d] = st.j[d] * ir0;
-        F[d] = st.F[d] * ir0;
-    }
-    sym_form(mnb, A);
-    const R zero[3] = {R(0.0f), R(0.0f), R(0.0f)};
-    if constexpr (HAS_LAM) {
-        R Qm[6], H[6];
-        sym_form(q, Qm);
-        sfor<6>([&](auto c) { H[c] = fma(R(0.5f), A[c], Qm[c]); });
-        sym_apply(H, F, zero, hF);
-        const R lin[3] = {fma(cst<R>(-2.0 / 3.0), q[4], fma(R(0.5f), hF[0], q[3])),
-                          fma(cst<R>(-2.0 / 3.0), q[6], fma(R(0.5f), hF[1], q[5])),
-                          fma(cst<R>(-2.0 / 3.0), q[8], fma(R(0.5f), hF[2], q[7]))};
-        sym_apply(Qm, j, lin, Fbar);
+        Xf<D3Q19>::forward(lam[0], P, Dd, Lm);
+        sfor<19>([&](auto k) { Db[k] = -Lm[k]; });
     } else {
-        R H[6];
-        sfor<6>([&](auto c) { H[c] = R(0.5f) * A[c]; });
-        sym_apply(H, F, zero, hF);
-        for (int d = 0; d < 3; ++d) Fbar[d] = R(0.5f) * hF[d];
+        sfor<19>([&](auto k) { Db[k] = R(0); });
     }
-    const R lin[3] = {cst<R>(-2.0 / 3.0) * mnb[4], cst<R>(-2.0 / 3.0) * mnb[6], cst<R>(-2.0 / 3.0) * mnb[8]};
-    sym_apply(A, j, lin, Aj);
-    // p' = lam + T^T (drho', j', mn')
-    mnb[0] = fma(R(11.0f), mnb[1], R(-3.0f) * mnb[2]);
-    mnb[3] = hF[0] - Aj[0];
-    mnb[5] = hF[1] - Aj[1];
-    mnb[7] = hF[2] - Aj[2];
-    Xf<D3Q19>::template backward<mask_all<D3Q19>()>(mnb, mu);
-    if constexpr (HAS_LAM) sfor<19>([&](auto i) { mu[i] = lam[i] + mu[i]; });
+    // s' and tau'
+    R sbar = Sbar[0] * st.B[0] + Sbar[1] * st.B[1] + Sbar[2] * st.B[2] + Sbar[3] * st.B[3] + Sbar[4] * st.B[4] +
+             Sbar[5] * st.B[5];
+    sfor<19>([&](auto k) {
+        if constexpr (D3Q19::viscous(CV(k))) sbar = fma(Db[k] * cst<R>(1.0 / norm2<D3Q19>(CV(k))), st.mn[k], sbar);
+    });
+    R sig[6];
+    sfor<6>([&](auto c) { sig[c] = Sbar[c]; });
+    if constexpr (CLOSURE != CL_NEWTON) {
+        const R taubar = taubar_d - sbar * st.s * st.s;
+        if (st.snorm > R(0)) {
+            const R c3 = a.smag_c3;
+            const R SB = strain_w_dot(st.S, st.B);
+            const R den = R(1) + R(2) * c3 * st.s * st.s * SB / st.snorm;
+            const R coef = taubar * c3 * R(2) / (st.snorm * den);
+            sfor<6>([&](auto c) { sig[c] = fma(coef * R(CV(c) < 3 ? 1 : 2), st.S[c], sig[c]); });
+        }
+    }
+    // mn' = Y^T(sigma) + D'_k s_k / |T_k|^2
+    R mnb[19];
+    sfor<19>([&](auto k) { mnb[k] = R(0); });
+    mnb[1] = -(a.s[1] * R(Eq<D3Q19>::YU_A) * ir0) * (sig[0] + sig[1] + sig[2]);
+    mnb[9] = st.s * ir0 * (R(-0.5) * sig[0] + R(0.25) * (sig[1] + sig[2]));
+    mnb[11] = st.s * ir0 * (R(0.75) * (sig[2] - sig[1]));
+    mnb[13] = st.s * ir0 * (R(-1.5) * sig[3]);
+    mnb[14] = st.s * ir0 * (R(-1.5) * sig[4]);
+    mnb[15] = st.s * ir0 * (R(-1.5) * sig[5]);
+    sfor<19>([&](auto k) {
+        if constexpr (!D3Q19::conserved(CV(k))) {
+            const R sk = D3Q19::viscous(CV(k)) ? st.s * cst<R>(1.0 / norm2<D3Q19>(CV(k))) : R(a.skn[k]);
+            mnb[k] = fma(Db[k], sk, mnb[k]);
+        }
+    });
+    // TF' and m_eq'
+    R TFb[19], meqb[19];
+    sfor<19>([&](auto k) {
+        constexpr double inv_n = 1.0 / norm2<D3Q19>(CV(k));
+        if constexpr (D3Q19::conserved(CV(k)))
+            TFb[k] = cst<R>(-inv_n) * Db[k];
+        else
+            TFb[k] = fma(R(0.5), mnb[k], cst<R>(-inv_n) * Db[k]);
+        meqb[k] = -mnb[k];
+    });
+    // j' = J^T m_eq' + sum_k TF'_k H_k F ;  F' = J^T TF' + j'/2
+    R jb[3], hF[3], jtf[3];
+    jt(st.j, meqb, ir0, jb);
+    {
+        // sum_k TF'_k H_k F = (J(F)^T TF') - (the j-independent rows 3..8 of J)^T TF'
+        jt(st.F, TFb, ir0, hF);
+        hF[0] -= TFb[3] - cst<R>(2.0 / 3.0) * TFb[4];
+        hF[1] -= TFb[5] - cst<R>(2.0 / 3.0) * TFb[6];
+        hF[2] -= TFb[7] - cst<R>(2.0 / 3.0) * TFb[8];
+    }
+    jt(st.j, TFb, ir0, jtf);
+    for (int d = 0; d < 3; ++d) {
+        jb[d] += hF[d];
+        Fbar[d] = fma(R(0.5), jb[d], jtf[d]);
+    }
+    // m' and p' = lam + T^T m'
+    R mb[19];
+    sfor<19>([&](auto k) { mb[k] = mnb[k]; });
+    mb[3] = jb[0];
+    mb[5] = jb[1];
+    mb[7] = jb[2];
+    const R drhob = R(-11) * meqb[1] + R(3) * meqb[2];
+    R back[19];
+    Xf<D3Q19>::template backward<mask_all_but_density<D3Q19>()>(mb, back);
+    sfor<19>([&](auto i) {
+        if constexpr (HAS_LAM)
+            mu[i] = lam[i] + (back[i] + drhob);
+        else
+            mu[i] = back[i] + drhob;
+    });
 }
 
 // ------------------------------------------------------------------------------------------
@@ -316,11 +308,11 @@ __device__ __forceinline__ void adjoint_unit(const AdjArgs<typename Store<ST>::R
     }
 }
 
-// Bound to 7 resident blocks per SM (72 registers): 128^3, T = 64, every state kept, 9.65 ms against 10.09 / 10.17 /
-// 10.44 at 8 / 9 / 6 blocks (8 spill 20 values; loading lambda again at the end instead of holding it, which
-// does without spills, 10.03 at 8).  Bound by HBM: 264 B a node and step at 86-90% of the copy bandwidth.
+// Bound to 8 resident blocks per SM (64 registers, a few spilled values): 128^3, T = 64, every state kept, 9.83 ms
+// against 9.92 at 7 (the reverse step waits on memory; more warps hide it).  Bound by HBM: 264 B a node and
+// step at 86-90% of the copy bandwidth.
 template <class ST, int CLOSURE>
-__global__ void __launch_bounds__(128, 7) k_adjoint_stream(const AdjArgs<typename Store<ST>::R> a0,
+__global__ void __launch_bounds__(128, 8) k_adjoint_stream(const AdjArgs<typename Store<ST>::R> a0,
                                                         const AdjArgs<typename Store<ST>::R> a1, const StreamCtl c) {
     stream_schedule(a0.st.ny, a0.st.nz, c, [&](int k, int z, int y0, int y1) {
         const long long es = -(long long)k * c.ring;

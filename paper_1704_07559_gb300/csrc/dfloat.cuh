@@ -7,9 +7,8 @@
 // floating-point technique for extending the available precision", Numer. Math. 18, 1971).  The pair is
 // not normalised after each operation: l stays within a few last places of h, so an operation is
 // exact to about 2^-44 of its operands' magnitude, 2^-20 of the last place of the float that is
-// stored in the end (normalising took 3 more
-// instructions an operation: lbm_init of a 192^3 FP32 box 15% longer).  Infinities and values beyond the FP32 range become NaN here; callers redo those
-// in FP64.
+// stored in the end (normalising took 3 more instructions an operation: lbm_init of a 192^3 FP32 box 15%
+// longer).  Infinities and values beyond the FP32 range become NaN here; callers redo those in FP64.
 #pragma once
 
 #include <stdint.h>
