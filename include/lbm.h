@@ -192,8 +192,8 @@ int lbm_step(lbm_ctx* ctx, int n);
  *                         than the GPU holds resident blocks; one launch per step otherwise (the
  *                         default).  On larger lattices, and on D2Q9 lattices, a step boundary
  *                         costs less than the multi-step launch's synchronisation.  FP32 D2Q9
- *                         lattices (not with the lagged closure, and with the power law up to 2^19
- *                         nodes) run four steps per launch in shared-memory tiles instead.
+ *                         lattices (not with the lagged closure, and with the power law, n != 1, up
+ *                         to 2^19 nodes) run four steps per launch in shared-memory tiles instead.
  *  LBM_SCHEDULE_PER_STEP  one launch per step.
  *  LBM_SCHEDULE_STREAM    several steps per launch wherever the storage allows it (not FP64),
  *                         whatever the lattice size.

@@ -15,7 +15,8 @@
 // 104 / 110, 4096^2 95.3 / 122 / 131; 256 threads (several passes a step, few warps) 22 at 256^2, 110 at 4096^2;
 // 64x32 120 at 4096^2, 6 steps 112, 2 steps 103 (32x16).  Smagorinsky 4096^2 94 / 98 / 105, deviatoric Chai 95 /
 // 106 / 112.  The power law is bound by its sweeps, which margins repeat: 512^2 42.1 / 48.7 / 51.8 but 1000^2
-// 70.2 / 63.5 / 67.2 and 4096^2 84 / 72 / 77, so it takes this form up to 2^19 nodes only.
+// 70.2 / 63.5 / 67.2 and 4096^2 84 / 72 / 77, so it takes this form up to 2^19 nodes only, unless n = 1 (no sweeps:
+// 4096^2 Yu 94.3 per step launch, 102.6; Chai 92.5, 95.7).
 #pragma once
 
 #include <atomic>
