@@ -31,7 +31,7 @@ cudaError_t launch_form(const StepArgs<typename Store<ST>::R>& a, cudaStream_t s
         // the lightest step: the plain grid always (1000^2, 2% of the threads idle: 97.4 GLUPS against 92.1 in
         // node order)
         dim3 b;
-        lattice_grid(a.nx, a.ny, a.nzc, &g, &b);
+        lattice_grid(a.nx, a.ny, a.nzc, &g, &b, T);
         return launch_pdl(k_step<L, ST, C, F, FO, true>, g, b, s, a, NodeMap{});
     } else {
         // rows that nearly fill their blocks keep the plain grid only where both buffers stay in L2 (121x89x38,

@@ -9,10 +9,10 @@ namespace lbm {
 template <class R>
 struct StepArgs;
 
-// geometry of a lattice launch: 128-thread blocks covering x (and several y rows when nx is small)
-inline void lattice_grid(int nx, int ny, int nz, dim3* grid, dim3* block) {
-    const int bx = nx <= 32 ? 32 : (nx <= 64 ? 64 : 128);
-    const int by = 128 / bx;
+// geometry of a lattice launch: blocks of `threads` covering x (and several y rows when nx is small)
+inline void lattice_grid(int nx, int ny, int nz, dim3* grid, dim3* block, int threads = 128) {
+    const int bx = nx <= 32 ? 32 : (nx <= 64 || threads <= 64 ? 64 : 128);
+    const int by = threads / bx;
     *block = dim3(bx, by, 1);
     *grid = dim3((nx + bx - 1) / bx, (ny + by - 1) / by, nz);
 }

@@ -1412,21 +1412,28 @@ inline NodeMap node_grid(const StepArgs<RS>& a, int threads, int waste, dim3* gr
     return g;
 }
 
-// One node per thread.  The bound names no minimum of resident blocks for the 3D lattices and
-// FP64: a minimum of one changes ptxas's register allocation (more registers, fewer resident
-// blocks).  FP32 D2Q9 is held to 16 blocks (32 registers, full occupancy; the power law spills up to 12
-// values there): 4096^2 power-law cavity, developed n = 0.5 flow, Yu / Chai 83.0 / 78.7 GLUPS, at 12 blocks
-// 79.8 / 76.8, at 10 71.3 / 68.2.
+// One node per thread.  The bound names no minimum of resident blocks for the 16-bit and FP32 3D lattices: a
+// minimum of one changes ptxas's register allocation (more registers, fewer resident blocks).  FP64 names one
+// that leaves it more registers than it takes unasked (128 in 3D, 64 in 2D): bound by the FP64 pipe, the step
+// gains by holding values instead of forming them again (GLUPS: D3Q19 channel Yu 1.28 -> 1.43, Newtonian box Chai
+// 2.11 -> 2.32, D3Q15 channel Yu 1.54 -> 1.63, 1000^2 D2Q9 Chai 4.88 -> 5.39; a cap of 80 in 3D 1.26).  FP32 D2Q9 is
+// held to 16 blocks (32 registers, full occupancy; the power law spills up to 12 values there): 4096^2
+// power-law cavity, developed n = 0.5 flow, Yu / Chai 83.0 / 78.7 GLUPS, at 12 blocks 79.8 / 76.8, at 10 71.3 / 68.2.
 template <class L, class ST>
 constexpr int step_min_blocks() {
-    return (L::Q == 9 && sizeof(ST) == 4) ? 16 : 0;
+    if (sizeof(ST) == 8) return L::Q == 9 ? 8 : 4;
+    return L::Q == 9 && sizeof(ST) == 4 ? 16 : 0;
 }
 
 template <class L, class ST, int CLOSURE, int FORMULA, bool FORCE, bool GRID>
 __global__ void __launch_bounds__(128, step_min_blocks<L, ST>())
     k_step(const StepArgs<typename Store<ST>::R> a, const NodeMap g) {
     pdl_wait();     // the previous step's stores are complete and visible from here on
-    pdl_release();  // every block has started: the next step may be scheduled into freed slots
+    // Every block has started: the next step may be scheduled into freed slots.  Not in FP64, whose blocks wait
+    // for their SM's share of the FP64 pipe: blocks of the next step that come early leave the rest to
+    // whichever SM is done first, and the SMs end up with unequal shares (40^3 1.85 against 2.39 GLUPS,
+    // 119x891 D2Q9 2.90 against 4.15).
+    if constexpr (sizeof(ST) != 8) pdl_release();
     int x, y, z;
     if (!(GRID ? node_in_grid<1>(a, x, y, z) : node_in_order<1>(a, g, x, y, z))) return;
     typename Store<ST>::R f[L::Q];
