@@ -353,6 +353,34 @@ struct Xf<D3Q19> {
         E[8] = t - a[14];
     }
 
+    // Even and odd parts of out_i = sum_k T_ki a_k over the non-conserved moments that are not viscous (1, 2, 4, 6,
+    // 8, 10, 12, 16, 17, 18): E0 for the rest population, E_p + O_p and E_p - O_p for pair p
+    template <class R>
+    static __device__ __forceinline__ void fixed_pairs(const R (&a)[19], R& E0, R (&E)[9], R (&O)[9]) {
+        E0 = fma(R(12.0f), a[2], R(-30.0f) * a[1]);
+        const R B1 = fma(R(-4.0f), a[2], R(-11.0f) * a[1]);  // axis pairs
+        const R B2 = fma(R(8.0f), a[1], a[2]);               // edge pairs
+        const R s = a[10] + a[12], t = a[10] - a[12];
+        E[0] = fma(R(-4.0f), a[10], B1);
+        E[1] = fma(R(2.0f), t, B1);
+        E[2] = fma(R(2.0f), s, B1);
+        E[3] = E[4] = B2 + s;
+        E[5] = E[6] = B2 + t;
+        E[7] = E[8] = fma(R(-2.0f), a[10], B2);
+        O[0] = R(-4.0f) * a[4];
+        O[1] = R(-4.0f) * a[6];
+        O[2] = R(-4.0f) * a[8];
+        const R u1 = a[4] + a[16], v1 = a[6] - a[17];
+        O[3] = v1 + u1;
+        O[4] = v1 - u1;
+        const R u2 = a[4] - a[16], v2 = a[8] + a[18];
+        O[5] = v2 + u2;
+        O[6] = v2 - u2;
+        const R u3 = a[6] + a[17], v3 = a[8] - a[18];
+        O[7] = v3 + u3;
+        O[8] = v3 - u3;
+    }
+
     template <class R>
     static __device__ __forceinline__ void forward(R f0, const R (&P)[9], const R (&D)[9], R (&m)[19]) {
         const R Exy = P[3] + P[4], Exz = P[5] + P[6], Eyz = P[7] + P[8];
@@ -492,6 +520,22 @@ struct Xf<D3Q15> {
         m[14] = w - x;
     }
 
+    // fixed_pairs of D3Q19 on this basis (moments 1, 2, 4, 6, 8, 14)
+    template <class R>
+    static __device__ __forceinline__ void fixed_pairs(const R (&a)[15], R& E0, R (&E)[7], R (&O)[7]) {
+        E0 = fma(R(16.0f), a[2], R(-2.0f) * a[1]);
+        E[0] = E[1] = E[2] = fma(R(-4.0f), a[2], -a[1]);
+        E[3] = E[4] = E[5] = E[6] = a[1] + a[2];
+        O[0] = R(-4.0f) * a[4];
+        O[1] = R(-4.0f) * a[6];
+        O[2] = R(-4.0f) * a[8];
+        const R p = a[8] + a[6], m = a[8] - a[6], c = a[4] + a[14], d = a[4] - a[14];
+        O[3] = p + c;
+        O[4] = p - c;
+        O[5] = m + d;
+        O[6] = m - d;
+    }
+
     // viscous_pairs from shared partial sums (moments 9..13)
     template <class R>
     static __device__ __forceinline__ void viscous_even(const R (&a)[15], R (&E)[7]) {
@@ -569,9 +613,8 @@ __host__ __device__ constexpr int second_moment(int cpt, int k) {
 // of the non-equilibrium distributions.  The contraction and T^-1 = T^t diag(1/|T_k|^2) are both
 // constant, so their product is formed at compile time: S_c = kS sum_k (sum_i c_i c_i T_ki) D_k with
 // D_k = s_k mn_k / |T_k|^2, in which only the energy moment and the viscous moments have nonzero sums.
-// Forming T^-1 L mn in the q directions and contracting it there, as the formula is written, made the
-// step one of instructions and registers: D3Q19 channel 256x128x128, 20 steps, FP32 39.1 GLUPS against
-// 41.7 in this form, FP16 44.2 against 51.3, D3Q15 BF16 54.3 against 59.6.
+// Forming T^-1 L mn in the q directions and contracting it there, as the formula is written (omega_split), made the
+// FP32 step one of instructions and registers: D3Q19 channel 256x128x128, 20 steps, 39.1 GLUPS against 41.7.
 template <class L, class R, class Take>
 __device__ __forceinline__ void chai_contract(const R (&D)[L::Q], R kS, Take take, R (&S)[L::NS]) {
     sfor<L::NS>([&](auto cpt) {
@@ -581,6 +624,51 @@ __device__ __forceinline__ void chai_contract(const R (&D)[L::Q], R kS, Take tak
         });
         S[cpt] = kS * acc;
     });
+}
+
+// The same formula as it is written, for S = A + s_nu B: Omega = T^-1 L mn of the rate-independent moments (by pairs
+// Ef0, Ef, Of) and of the viscous ones (Ev; both velocities of a pair get the same), contracted with c c, to
+// which odd parts add nothing.  Lattices with a closure and 16-bit storage step by this one: the folded product
+// rounds S differently in its last FP32 place, and where that moves a population across a rounding
+// boundary of the storage the neighbours follow, until after some 20 steps the states are a storage
+// rounding apart everywhere (D3Q15 BF16 channel 256x128x128: 5e-3 of the state, which is also how far
+// either is from 64 bits).  The off-diagonal rate-independent sums cancel exactly (the two edge or four corner pairs
+// involved hold the same value), and the factor 2 of a pair's two velocities is exact in kS2 = 2 kS.
+template <class L, int CPT, class R>
+__device__ __forceinline__ R contract_pairs(const R (&E)[L::NP]) {
+    constexpr int a = strain_axis<L>(CPT, 0), b = strain_axis<L>(CPT, 1);
+    R acc = nzero<R>();
+    sfor<L::NP>([&](auto p) { acc = cadd<L::c(L::pa(CV(p)), a) * L::c(L::pa(CV(p)), b)>(acc, E[p]); });
+    return acc;
+}
+template <class L, class RS, class R>
+__device__ __forceinline__ void omega_split(const StepArgs<RS>& a, const R (&mn)[L::Q], R ir0, R& Ef0, R (&Ef)[L::NP],
+                                            R (&Of)[L::NP], R (&Ev)[L::NP], R (&A)[L::NS], R (&B)[L::NS]) {
+    const R kS2 = R(-3.0f) * ir0;
+    R D[L::Q];
+    sfor<L::Q>([&](auto k) {
+        if constexpr (L::viscous(CV(k)))
+            D[k] = cst<R>(1.0 / norm2<L>(CV(k))) * mn[k];
+        else if constexpr (!L::conserved(CV(k)))
+            D[k] = R(a.skn[k]) * mn[k];
+    });
+    Xf<L>::fixed_pairs(D, Ef0, Ef, Of);
+    Xf<L>::viscous_even(D, Ev);
+    sfor<L::NS>([&](auto c) {
+        if constexpr (CV(c) < L::D)
+            A[c] = kS2 * contract_pairs<L, CV(c)>(Ef);
+        else
+            A[c] = R(0.0f);
+        B[c] = kS2 * contract_pairs<L, CV(c)>(Ev);
+    });
+}
+// S:T of a diagonal S
+template <class L, class R>
+__device__ __forceinline__ R diag_dot(const R (&S)[L::NS], const R (&T)[L::NS]) {
+    if constexpr (L::NS == 6)
+        return fma(S[0], T[0], fma(S[1], T[1], S[2] * T[2]));
+    else
+        return fma(S[0], T[0], S[1] * T[1]);
 }
 
 // ------------------------------------------------------------------------------------------
@@ -1352,14 +1440,73 @@ __device__ __forceinline__ void collide(const StepArgs<typename Store<ST>::R>& a
     sfor<Q>([&](auto i) { sink(i, f[i] - out[i]); });
 }
 
+// The Guo-type discrete force in opposite-pair form (noneq_pairs): even parts E, c.F of each pair (odd part 3 w c.F)
+// and u.F (rest -3 w0 u.F)
+template <class L, class R>
+__device__ __forceinline__ void force_pairs(const R (&u)[3], const R (&F)[3], R& uF, R (&E)[L::NP], R (&cF)[L::NP]) {
+    uF = fma(u[0], F[0], fma(u[1], F[1], u[2] * F[2]));
+    sfor<L::NP>([&](auto p) {
+        constexpr int i = L::pa(CV(p));
+        constexpr int cx = L::c(i, 0), cy = L::c(i, 1), cz = L::c(i, 2);
+        constexpr double w = double(L::wnum(i)) / L::WDEN;
+        const R cu = cadd<cz>(cadd<cy>(cadd<cx>(nzero<R>(), u[0]), u[1]), u[2]);
+        cF[p] = cadd<cz>(cadd<cy>(cadd<cx>(nzero<R>(), F[0]), F[1]), F[2]);
+        E[p] = fma(cst<R>(9.0 * w) * cu, cF[p], cst<R>(-3.0 * w) * uF);
+    });
+}
+
+// Chai's route of a 16-bit lattice at one node (nx odd; step_pair.cuh has the pair): as collide, with Omega formed
+// in the q directions (omega_split), f* = f - Omega + Fbar.
+template <class L, class ST, int CLOSURE, bool FORCE, class Sink>
+__device__ __forceinline__ void collide_omega(const StepArgs<typename Store<ST>::R>& a,
+                                              typename Store<ST>::R (&f)[L::Q], int node, Sink&& sink) {
+    using R = typename Store<ST>::R;
+    constexpr int Q = L::Q, NS = L::NS, NP = L::NP;
+    R P[NP], Dd[NP], F[3];
+    pair_sums<L>(f, P, Dd);
+    node_force<L, FORCE>(a, node, F);
+    const R ir0 = R(a.inv_rho0);
+    R drho, j[3], u[3], m[Q], mn[Q], fn0, Pn[NP], Dn[NP];
+    conserved_moments<L, F_CHAI, FORCE>(f[0], P, Dd, F, ir0, drho, j, u, m);
+    noneq_pairs<L, FORCE>(f[0], P, Dd, drho, j, u, F, fn0, Pn, Dn);
+    Xf<L>::forward(fn0, Pn, Dn, mn);
+    constexpr double w0 = double(L::wnum(0)) / L::WDEN;
+    R uF, FE[NP], cF[NP];
+    if constexpr (FORCE) force_pairs<L>(u, F, uF, FE, cF);
+    R Ef0, Ef[NP], Of[NP], Ev[NP], A[NS], B[NS], S[NS], snu;
+    omega_split<L>(a, mn, ir0, Ef0, Ef, Of, Ev, A, B);
+    // everything but s_nu Omega_v is folded into f now, so that only f and Omega_v stay live across the closure
+    f[0] -= Ef0;
+    if constexpr (FORCE) f[0] = fma(cst<R>(-3.0 * w0), uF, f[0]);
+    sfor<NP>([&](auto p) {
+        R e = Ef[p], o = Of[p];
+        if constexpr (FORCE) {
+            constexpr double w = double(L::wnum(L::pa(CV(p)))) / L::WDEN;
+            e -= FE[p];
+            o = fma(cst<R>(-3.0 * w), cF[p], o);
+        }
+        f[L::pa(CV(p))] -= e + o;
+        f[L::pb(CV(p))] -= e - o;
+    });
+    solve_tau<L, R, CLOSURE, true>(A, B, a, S, snu, node);
+    sink(std::integral_constant<int, 0>{}, f[0]);
+    sfor<NP>([&](auto p) {
+        const R e = snu * Ev[p];
+        sink(std::integral_constant<int, L::pa(CV(p))>{}, f[L::pa(CV(p))] - e);
+        sink(std::integral_constant<int, L::pb(CV(p))>{}, f[L::pb(CV(p))] - e);
+    });
+}
+
 // The collision with f* stored at the node.  ds shifts the populations' destination by that many elements (a
 // launch that writes each step to its own buffer of a ring); the pull's es does the same for the source.
 template <class L, class ST, int CLOSURE, int FORMULA, bool FORCE>
 __device__ __forceinline__ void step_body(const StepArgs<typename Store<ST>::R>& a, typename Store<ST>::R (&f)[L::Q],
                                           int node, long long ds = 0) {
-    collide<L, ST, CLOSURE, FORMULA, FORCE>(a, f, node, [&](auto i, auto v) {
-        Store<ST>::st(static_cast<ST*>(a.dstp[CV(i)]) + ds + node, v);
-    });
+    auto sink = [&](auto i, auto v) { Store<ST>::st(static_cast<ST*>(a.dstp[CV(i)]) + ds + node, v); };
+    if constexpr (sizeof(ST) == 2 && FORMULA == F_CHAI && CLOSURE != CL_NEWTON)
+        collide_omega<L, ST, CLOSURE, FORCE>(a, f, node, sink);
+    else
+        collide<L, ST, CLOSURE, FORMULA, FORCE>(a, f, node, sink);
 }
 
 // Which node(s) a thread takes: PER x-adjacent nodes each (nx a multiple of PER), in node order over the

@@ -42,12 +42,13 @@ __device__ __forceinline__ V2& operator-=(V2& a, V2 b) { return a = a - b; }
 __device__ __forceinline__ V2 fma(V2 a, V2 b, V2 c) { return V2(__ffma2_rn(a.v, b.v, c.v)); }
 
 // Smagorinsky closure for the pair: the quadratic form of |S|^2 in s = 1/tau is formed for both lanes at
-// once, then each lane runs the scalar fixed point of step.cuh.
-template <class L, int CLOSURE>
+// once, then each lane runs the scalar fixed point of step.cuh.  DIAG: A is diagonal.
+template <class L, int CLOSURE, bool DIAG>
 __device__ __forceinline__ void solve_tau_pair(const V2 (&A)[L::NS], const V2 (&B)[L::NS], const StepArgs<float>& a,
                                               V2& snu) {
     static_assert(CLOSURE == CL_SMAG, "16-bit storage builds this closure and fixed rates");
-    const V2 qa = strain_dot<L>(A, A), qb2 = V2(2.0f) * strain_dot<L>(A, B), qc = strain_dot<L>(B, B);
+    const V2 qa = DIAG ? diag_dot<L>(A, A) : strain_dot<L>(A, A);
+    const V2 qb2 = V2(2.0f) * (DIAG ? diag_dot<L>(A, B) : strain_dot<L>(A, B)), qc = strain_dot<L>(B, B);
     const float t0 = tau_fixed_point<CLOSURE>(qa.lo(), qb2.lo(), qc.lo(), a);
     const float t1 = tau_fixed_point<CLOSURE>(qa.hi(), qb2.hi(), qc.hi(), a);
     snu = V2(c_rcp(t0), c_rcp(t1));
@@ -131,7 +132,7 @@ __device__ __forceinline__ void step_pair(const StepArgs<float>& a, const F2 (&f
         if constexpr (CLOSURE != CL_NEWTON) {
             R A[NS], B[NS];
             Eq<L>::yu_split(mn, R(a.s[1] * float(Eq<L>::YU_A)) * ir0, ir0, A, B);
-            solve_tau_pair<L, CLOSURE>(A, B, a, snu);
+            solve_tau_pair<L, CLOSURE, false>(A, B, a, snu);
             sfor<Q>([&](auto k) {
                 if constexpr (L::viscous(CV(k))) {
                     constexpr double inv_n = 1.0 / norm2<L>(CV(k));
@@ -141,7 +142,7 @@ __device__ __forceinline__ void step_pair(const StepArgs<float>& a, const F2 (&f
         }
     } else {
         // Chai route: the non-equilibrium distributions f - f_eq + Fbar/2 (opposite-pair form), their
-        // moments mn = T fn, and S from them with the contraction folded into T^-1 (chai_contract).
+        // moments mn = T fn, and S from Omega = T^-1 L mn in the q directions (omega_split).
         // The post-collision state is formed from the same mn as f* = T^-1 m*, m*_k = m_eq_k + TF_k/2 +
         // (1 - s_k) mn_k (the moments of f are mn + m_eq - TF/2), so neither f nor fn has to stay live.
         drho = f[0];
@@ -158,8 +159,9 @@ __device__ __forceinline__ void step_pair(const StepArgs<float>& a, const F2 (&f
             noneq_pairs<L, FORCE>(f[0], P, Dd, drho, j, u, F, fn0, Pn, Dn);
             Xf<L>::forward(fn0, Pn, Dn, mn);
         }
+        R Ef0, Ef[NP], Of[NP], Ev[NP], A[NS], B[NS];
+        omega_split<L>(a, mn, ir0, Ef0, Ef, Of, Ev, A, B);
         // G_k of the rate-independent moments before the closure, as on the Yu route
-        R Dn[Q];
         {
             R meq[Q], TF[Q];
             Eq<L>::meq(drho, j, u, meq);
@@ -167,27 +169,20 @@ __device__ __forceinline__ void step_pair(const StepArgs<float>& a, const F2 (&f
             sfor<Q>([&](auto k) {
                 constexpr double inv_n = 1.0 / norm2<L>(CV(k));
                 constexpr bool has_tf = FORCE && !Eq<L>::ghost(CV(k)) && CV(k) != 0;
-                if constexpr (L::viscous(CV(k))) {
-                    Dn[k] = cst<R>(inv_n) * mn[k];
-                } else if constexpr (!L::conserved(CV(k))) {
-                    Dn[k] = R(a.skn[k]) * mn[k];
-                }
                 // m_k + TF_k = mn_k + m_eq_k + TF_k / 2
-                R base = Eq<L>::ghost(CV(k)) ? mn[k] : (L::conserved(CV(k)) ? meq[k] : mn[k] + meq[k]);
+                R base = Eq<L>::ghost(CV(k)) ? mn[k] : mn[k] + meq[k];
                 if constexpr (has_tf) base = fma(R(0.5f), TF[k], base);
+                base = cst<R>(inv_n) * base;
                 if constexpr (L::conserved(CV(k)) || L::viscous(CV(k)))
-                    G[k] = cst<R>(inv_n) * base;
+                    G[k] = base;
                 else
-                    G[k] = fma(cst<R>(inv_n), base, -Dn[k]);
+                    G[k] = fma(R(-a.skn[k]), mn[k], base);
             });
         }
-        const R kS = R(-1.5f) * ir0;
-        R A[NS], B[NS];
-        chai_contract<L>(Dn, kS, [](int k) { return !L::conserved(k) && !L::viscous(k); }, A);
-        chai_contract<L>(Dn, kS, [](int k) { return L::viscous(k); }, B);
-        solve_tau_pair<L, CLOSURE>(A, B, a, snu);
+        solve_tau_pair<L, CLOSURE, true>(A, B, a, snu);
         sfor<Q>([&](auto k) {
-            if constexpr (L::viscous(CV(k))) G[k] = fma(-snu, Dn[k], G[k]);
+            constexpr double inv_n = 1.0 / norm2<L>(CV(k));
+            if constexpr (L::viscous(CV(k))) G[k] = fma(-(snu * cst<R>(inv_n)), mn[k], G[k]);
         });
     }
     R fs[Q];
