@@ -97,6 +97,9 @@ __device__ __forceinline__ X init_tau(const StepArgs<double>& a, const InitConst
     });
     const X n = XC<X>::root(X(2.0f) * ss + sh);  // |rho0 S|, |S| = sqrt(2 S:S)
     if (k.closure == CL_POWERLAW) {
+        // a pair whose squares left the FP32 range: no clamp may hide it, the node is redone in FP64
+        if constexpr (!std::is_same<X, double>::value)
+            if (!(XC<X>::full(n) <= 3.0e38)) return X(nanf(""));
         double t = 0.5 + a.pl_k3 * pow(XC<X>::full(n) * a.inv_rho0, a.pl_nm1);
         if (!(t >= a.pl_tau_min)) t = a.pl_tau_min;
         if (t > a.pl_tau_max) t = a.pl_tau_max;
