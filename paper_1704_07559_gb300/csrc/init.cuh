@@ -95,11 +95,15 @@ __device__ __forceinline__ X init_tau(const StepArgs<double>& a, const InitConst
             sh = fma(g, g, sh);
         }
     });
-    const X n = XC<X>::root(X(2.0f) * ss + sh);  // |rho0 S|, |S| = sqrt(2 S:S)
+    const X n2 = X(2.0f) * ss + sh, n = XC<X>::root(n2);  // |rho0 S|, |S| = sqrt(2 S:S)
     if (k.closure == CL_POWERLAW) {
-        // a pair whose squares left the FP32 range: no clamp may hide it, the node is redone in FP64
-        if constexpr (!std::is_same<X, double>::value)
-            if (!(XC<X>::full(n) <= 3.0e38)) return X(nanf(""));
+        // a pair whose squares left the FP32 range, or lost bits below it (tau follows log |S| down to any strain, and
+        // only gradients that are zero give zero): no clamp may hide it, the node is redone in FP64
+        if constexpr (!std::is_same<X, double>::value) {
+            float g = 0.0f;
+            sfor<L::D>([&](auto p) { sfor<L::D>([&](auto q) { g = fmaxf(g, fabsf(G[CV(p)][CV(q)].h)); }); });
+            if (!(XC<X>::full(n) <= 3.0e38) || (n2.h < 0x1p-100f && g > 0.0f)) return X(nanf(""));
+        }
         double t = 0.5 + a.pl_k3 * pow(XC<X>::full(n) * a.inv_rho0, a.pl_nm1);
         if (!(t >= a.pl_tau_min)) t = a.pl_tau_min;
         if (t > a.pl_tau_max) t = a.pl_tau_max;

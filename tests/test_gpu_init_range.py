@@ -36,3 +36,14 @@ def test_power_law_with_huge_gradients(q, dims, n, size):
     g[0, :, 2, 1::7] = -size
     a, b = states(q, dims, np.zeros(shape), np.zeros((d,) + shape), g, closure="powerlaw", pl_n=n, pl_k=0.02)
     assert np.all(np.isfinite(b)) and close(a, b)
+
+
+@pytest.mark.parametrize("q,dims", [(19, (33, 4, 3)), (15, (20, 3, 3)), (9, (40, 5, 1))])
+@pytest.mark.parametrize("n,K", [(0.95, 0.116), (1.05, 1.0), (0.98, 0.3)])
+def test_power_law_with_tiny_gradients(q, dims, n, K):
+    d = 2 if q == 9 else 3
+    shape = dims[::-1]
+    rng = np.random.default_rng(2)
+    g = rng.standard_normal((d * d,) + shape) * 10.0 ** rng.uniform(-26, -12, size=shape)
+    a, b = states(q, dims, np.zeros(shape), np.zeros((d,) + shape), g, closure="powerlaw", pl_n=n, pl_k=K)
+    assert close(a, b)
