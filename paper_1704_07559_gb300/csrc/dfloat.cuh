@@ -8,7 +8,8 @@
 // not normalised after each operation: l stays within a few last places of h, so an operation is
 // exact to about 2^-44 of its operands' magnitude, 2^-20 of the last place of the float that is
 // stored in the end (normalising took 3 more instructions an operation: lbm_init of a 192^3 FP32 box 15%
-// longer).  Infinities and values beyond the FP32 range become NaN here; callers redo those in FP64.
+// longer).  Infinities and values beyond the FP32 range become NaN here, and values below about 2^-100 lose the last
+// bits of their low part; callers redo both in FP64.
 #pragma once
 
 #include <stdint.h>

@@ -13,7 +13,8 @@
 // 5.9 ms for a 192^3 FP32 box with a gradient, now 0.35 ms (its bytes take 0.19 ms at the measured copy
 // bandwidth; the error against 64 bits is unchanged, 2.5e-8).  FP64 storage runs the pair form above in FP64; the other storages run it in
 // pairs of floats (dfloat.cuh: 48 bits, rounded once to FP32 at the end, as the FP64 result was), and
-// only nodes next to a moving wall or with a result that is not finite repeat it in FP64.
+// only nodes next to a moving wall, with a result that is not finite or with values near the smallest of FP32
+// repeat it in FP64.
 #pragma once
 
 #include "dfloat.cuh"
@@ -238,7 +239,7 @@ __device__ __forceinline__ void unstream(const StepArgs<double>& a, int x, int y
     });
 }
 
-// One node in arithmetic X: loads, populations, tau; returns whether every result is finite (in FP64
+// One node in arithmetic X: loads, populations, tau; returns whether X holds every result (in FP64
 // always true: its infinities and NaN are the result).
 template <class L, class ST, bool FORCE, class X, class V>
 __device__ __forceinline__ bool init_at(const StepArgs<double>& a, const InitConst<X>& k, int node,
@@ -277,12 +278,14 @@ __device__ __forceinline__ bool init_at(const StepArgs<double>& a, const InitCon
     tau_out = XC<X>::template out<V>(tau);
     init_node<L, FORCE>(k, dr, j, F, gu != nullptr, G, tau, f);
     if constexpr (std::is_same<X, double>::value) return true;
-    V s = tau_out;
+    V s = V(0);
     sfor<L::Q>([&](auto i) { s += r_abs(f[i]); });
-    return s < V(3.0e38f);  // false for NaN too
+    // false for NaN too; below 2^-90 a pair's low part, 2^-24 to 2^-48 of the value, comes near the smallest FP32
+    // numbers and loses bits
+    return s + tau_out < V(3.0e38f) && (s >= V(0x1p-90f) || s == V(0));
 }
 
-// the node in FP64 up to the stores: float pairs that left the FP32 range on the way, and nodes next to
+// the node in FP64 up to the stores: float pairs that left the FP32 range on the way, at either end, and nodes next to
 // a moving wall, whose term joins the population before it is rounded
 template <class L, class ST, bool FORCE>
 __device__ __noinline__ void init_again(const StepArgs<double>& a, const InitConst<double>& k, int x, int y, int z,

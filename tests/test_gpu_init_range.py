@@ -47,3 +47,18 @@ def test_power_law_with_tiny_gradients(q, dims, n, K):
     g = rng.standard_normal((d * d,) + shape) * 10.0 ** rng.uniform(-26, -12, size=shape)
     a, b = states(q, dims, np.zeros(shape), np.zeros((d,) + shape), g, closure="powerlaw", pl_n=n, pl_k=K)
     assert close(a, b)
+
+
+@pytest.mark.parametrize("q,dims", [(19, (33, 14, 13)), (9, (140, 45, 1))])
+@pytest.mark.parametrize("closure", ["newton", "smag"])
+@pytest.mark.parametrize("gradient", [False, True])
+def test_values_below_the_pairs_range_are_rounded_once(q, dims, closure, gradient):
+    """Nodes whose values all lie below 2^-103, where a pair's low part is subnormal: bit for bit the FP64 result."""
+    d = 2 if q == 9 else 3
+    shape = dims[::-1]
+    rng = np.random.default_rng(4)
+    size = 10.0 ** rng.uniform(-36, -33, size=shape)
+    drho, u = rng.standard_normal(shape) * size, rng.standard_normal((d,) + shape) * size
+    g = rng.standard_normal((d * d,) + shape) * size if gradient else None
+    a, b = states(q, dims, drho, u, g, closure=closure, smag_cs=0.17)
+    assert np.array_equal(a.view(np.int32), b.view(np.int32)), int((a != b).sum())
