@@ -159,10 +159,12 @@ struct Store<__nv_bfloat16> {
 __device__ __forceinline__ float r_abs(float x) { return fabsf(x); }
 __device__ __forceinline__ double r_abs(double x) { return fabs(x); }
 // Closure arithmetic: in FP32 the approximate reciprocal, reciprocal square root, logarithm and power of
-// two (errors of a few ulp, far inside the FP32 tolerance of S), in FP64 the IEEE operations.  The FP32
-// ones are the instructions that take subnormals as zero, without the scaling around them (channel
+// two (errors of a few ulp, far inside the FP32 tolerance of S), in FP64 the IEEE operations.  The reciprocal and the
+// square root are the instructions that take subnormals as zero, without the scaling around them (channel
 // 256x128x128, 20 steps, Smagorinsky: FP16 Yu 61.1 -> 64.1 GLUPS, Chai 51.3 -> 53.8, FP32 Chai 41.7 -> 42.1):
-// tau lies above 1/2, and a squared strain below 2^-126 counts as zero.
+// tau lies above 1/2, and a strain under 1.1e-19, whose square is subnormal, adds less than half a last place to
+// a tau0 of 1/2 and more for any 3 Cs^2 below 2.7e11.  The logarithm is not: tau of the power law follows log |S| down
+// to any strain.
 __device__ __forceinline__ float c_rcp(float x) {
     float y;
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
@@ -175,14 +177,10 @@ __device__ __forceinline__ float c_sqrt(float x) {
     return x >= 1.17549435e-38f ? x * y : 0.0f;
 }
 __device__ __forceinline__ double c_sqrt(double x) { return sqrt(x); }
-__device__ __forceinline__ float c_log2(float x) {
-    float y;
-    asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-    return y;
-}
+__device__ __forceinline__ float c_log2(float x) { return __log2f(x); }
 __device__ __forceinline__ float c_exp2(float x) {
     float y;
-    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    asm("ex2.approx.f32 %0, %1;" : "=f"(y) : "f"(x));
     return y;
 }
 // |S|^(n-1) of the power-law closure from q2 = 2 S:S = |S|^2: in FP32 one fast power of q2 with
