@@ -65,12 +65,13 @@ __device__ __forceinline__ void pull_tile(const StepArgs<float>& a, const float*
     });
 }
 
-// position p of an axis of n nodes: wrapped on a periodic axis, as it is on an axis with walls
-__device__ __forceinline__ int wrap_pos(int p, int n, bool walls) {
-    if (walls) return p;
-    while (p < 0) p += n;
-    while (p >= n) p -= n;
-    return p;
+// Position p of a periodic axis of n nodes, wrapped.  A tile reaches less than its own extent beyond the lattice, so
+// one step of n is enough unless the axis is shorter than that; a loop for every node instead cost more
+// than the tiles gained on periodic lattices (4096^2 Newtonian Yu, 172 us a step with it, 129 without).
+template <int EXTENT>
+__device__ __forceinline__ int wrap_pos(int p, int n) {
+    if (n < EXTENT) return p < 0 ? n - 1 - (-1 - p) % n : p % n;
+    return p < 0 ? p + n : (p >= n ? p - n : p);
 }
 
 template <class L, int CLOSURE, int FORMULA, bool FORCE, int BH>
@@ -89,7 +90,7 @@ __global__ void __launch_bounds__(BLOCK_THREADS) k_step_block(const StepArgs<flo
         float* to = sm + (CV(k) & 1) * 9 * PITCH;
         for (int t = threadIdx.x; t < W * H; t += BLOCK_THREADS) {
             const int ly = t / W + CV(k), lx = t - (t / W) * W + CV(k);
-            const int x = wrap_pos(ox + lx, a.nx, wx), y = wrap_pos(oy + ly, a.ny, wy);
+            const int x = wx ? ox + lx : wrap_pos<SW>(ox + lx, a.nx), y = wy ? oy + ly : wrap_pos<SH>(oy + ly, a.ny);
             bool mine = x >= 0 && x < a.nx && y >= 0 && y < a.ny;  // false only beyond a wall
             if (LAST) mine = mine && ox + lx < a.nx && oy + ly < a.ny;  // and past a ragged end
             if (!mine) continue;
