@@ -9,7 +9,7 @@
 // another; a margin ends at a wall, where the pull reflects the node's own populations.  Every node update is
 // the one-step kernel's, so the state equals one launch per step bit for bit.
 //
-// Tile: 32 x 20, so that the first step's 38 x 26 nodes take one pass of 1024 threads (64 registers; 1.27 node
+// Tile: 32 x 20, so that the first step's 38 x 26 nodes take one pass of 1024 threads (1.27 node
 // updates computed per one kept); 32 x 16 (1.31) where 32 x 20 leaves SMs without a tile.  Measured (Newtonian
 // Yu, GLUPS per step launch / 32x16 / 32x20): 256^2 21.5 / 38.6 / 36.5, 512^2 56.9 / 72.7 / 75.8, 1000^2 98.9 /
 // 104 / 110, 4096^2 95.3 / 122 / 131; 256 threads (several passes a step, few warps) 22 at 256^2, 110 at 4096^2;
@@ -17,6 +17,11 @@
 // 106 / 112.  The power law is bound by its sweeps, which margins repeat: 512^2 42.1 / 48.7 / 51.8 but 1000^2
 // 70.2 / 63.5 / 67.2 and 4096^2 84 / 72 / 77, so it takes this form up to 2^19 nodes only, unless n = 1 (no sweeps:
 // 4096^2 Yu 94.3 per step launch, 102.6; Chai 92.5, 95.7).
+//
+// The bound keeps two blocks on an SM (32 registers).  Every form but the forced power law and the forced deviatoric
+// closure takes 32 anyway; those took 42 to 47, one block a SM, and were slower than one launch per step (forced
+// cavity 4096^2, us a step, one block / two / per step: deviatoric Yu 207 / 165 / 180, Chai 217 / 179 / 185; power
+// law n = 0.5, 700^2 Yu 10.9 / 9.7 / 9.5, with 52 bytes spilled).
 #pragma once
 
 #include <atomic>
@@ -67,7 +72,7 @@ __device__ __forceinline__ void pull_tile(const StepArgs<float>& a, const float*
 
 // Position p of a periodic axis of n nodes, wrapped.  A tile reaches less than its own extent beyond the lattice, so
 // one step of n is enough unless the axis is shorter than that; a loop for every node instead cost more
-// than the tiles gained on periodic lattices (4096^2 Newtonian Yu, 172 us a step with it, 129 without).
+// than the tiles gained on periodic lattices (4096^2 Newtonian Yu, 172 us a step with it, 139 without, 175 one by one).
 template <int EXTENT>
 __device__ __forceinline__ int wrap_pos(int p, int n) {
     if (n < EXTENT) return p < 0 ? n - 1 - (-1 - p) % n : p % n;
@@ -75,7 +80,7 @@ __device__ __forceinline__ int wrap_pos(int p, int n) {
 }
 
 template <class L, int CLOSURE, int FORMULA, bool FORCE, int BH>
-__global__ void __launch_bounds__(BLOCK_THREADS) k_step_block(const StepArgs<float> a) {
+__global__ void __launch_bounds__(BLOCK_THREADS, 2) k_step_block(const StepArgs<float> a) {
     constexpr int SH = tile_rows(BH), PITCH = SW * SH;
     extern __shared__ float sm[];
     pdl_wait();
