@@ -271,12 +271,6 @@ cudaError_t run_step(const lbm_ctx* c, const void* src, void* dst) {
     return c->p.precision == LBM_FP64 ? step_between<double>(c, src, dst) : step_between<float>(c, src, dst);
 }
 
-// Whether the next steps may run BLOCK_STEPS to a launch (step_block.cuh): FP32 D2Q9 on the automatic schedule
-bool use_blocks(const lbm_ctx* c, int steps_left) {
-    return c->q == 9 && c->p.precision == LBM_FP32 && c->schedule == LBM_SCHEDULE_AUTO &&
-           steps_left >= lbm::BLOCK_STEPS;
-}
-
 // n steps from the current buffer, one or (D2Q9) BLOCK_STEPS per launch, from two sets of arguments filled once:
 // a small lattice's step is no longer than what the host does between two launches
 template <class R>
@@ -287,19 +281,17 @@ cudaError_t step_by_step(lbm_ctx* c, int n, long long* launches) {
     set_buffers(c, &a[0], c->buf[0], c->buf[1]);
     set_buffers(c, &a[1], c->buf[1], c->buf[0]);
     const int force = has_force(c) ? 1 : 0;
+    bool blocks = false;  // BLOCK_STEPS to a launch (step_block.cuh): FP32 D2Q9 on the automatic schedule
+    if constexpr (std::is_same<R, float>::value)
+        blocks = c->q == 9 && c->schedule == LBM_SCHEDULE_AUTO && n >= lbm::BLOCK_STEPS &&
+                 lbm::block_d2q9_f32_pays(a[0], c->p.closure, force);
     for (int it = 0; it < n;) {
-        int k = 1;
-        cudaError_t e = cudaErrorNotSupported;
+        const int k = blocks && n - it >= lbm::BLOCK_STEPS ? lbm::BLOCK_STEPS : 1;
+        cudaError_t e = cudaErrorInvalidValue;
         if constexpr (std::is_same<R, float>::value) {
-            if (use_blocks(c, n - it)) {
-                e = lbm::block_d2q9_f32(a[c->cur], c->p.closure, c->p.formula, force, c->stream);
-                k = lbm::BLOCK_STEPS;
-            }
+            if (k > 1) e = lbm::block_d2q9_f32(a[c->cur], c->p.closure, c->p.formula, force, c->stream);
         }
-        if (e == cudaErrorNotSupported) {
-            e = launch_step(c, a[c->cur], force);
-            k = 1;
-        }
+        if (k == 1) e = launch_step(c, a[c->cur], force);
         if (e != cudaSuccess) return e;
         c->cur = 1 - c->cur;
         it += k;

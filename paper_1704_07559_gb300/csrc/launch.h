@@ -123,9 +123,9 @@ LBM_DECLARE_STREAM_ENTRY(d3q15_f16, float)
 LBM_DECLARE_STREAM_ENTRY(d3q15_bf16, float)
 LBM_DECLARE_STREAM_ENTRY(d2q9_f32, float)
 #undef LBM_DECLARE_STREAM_ENTRY
-// BLOCK_STEPS steps per launch in shared-memory tiles (step_block.cuh); cudaErrorNotSupported where it does
-// not apply or pay, the caller then steps one by one
+// BLOCK_STEPS steps per launch in shared-memory tiles (step_block.cuh), and whether that is the faster form
 constexpr int BLOCK_STEPS = 4;
+bool block_d2q9_f32_pays(const StepArgs<float>& a, int closure, int force);
 cudaError_t block_d2q9_f32(const StepArgs<float>& a, int closure, int formula, int force, cudaStream_t s);
 // ring launches (each step writes a buffer of its own): D3Q19 FP32, Newtonian and Smagorinsky
 cudaError_t stream_ring_d3q19_f32(const StepArgs<float>& a, const StreamCtl& c, int closure, int formula, int force,

@@ -13,10 +13,7 @@
 // updates computed per one kept); 32 x 16 (1.31) where 32 x 20 leaves SMs without a tile.  Measured (Newtonian
 // Yu, GLUPS per step launch / 32x16 / 32x20): 256^2 21.5 / 38.6 / 36.5, 512^2 56.9 / 72.7 / 75.8, 1000^2 98.9 /
 // 104 / 110, 4096^2 95.3 / 122 / 131; 256 threads (several passes a step, few warps) 22 at 256^2, 110 at 4096^2;
-// 64x32 120 at 4096^2, 6 steps 112, 2 steps 103 (32x16).  Smagorinsky 4096^2 94 / 98 / 105, deviatoric Chai 95 /
-// 106 / 112.  The power law is bound by its sweeps, which margins repeat: 512^2 42.1 / 48.7 / 51.8 but 1000^2
-// 70.2 / 63.5 / 67.2 and 4096^2 84 / 72 / 77, so it takes this form up to 2^19 nodes only, unless n = 1 (no sweeps:
-// 4096^2 Yu 94.3 per step launch, 102.6; Chai 92.5, 95.7).
+// 64x32 120 at 4096^2, 6 steps 112, 2 steps 103 (32x16).  Where tiles are taken: block_pays.
 //
 // The bound keeps two blocks on an SM (32 registers).  Every form but the forced power law and the forced deviatoric
 // closure takes 32 anyway; those took 42 to 47, one block a SM, and were slower than one launch per step (forced
@@ -113,6 +110,37 @@ __global__ void __launch_bounds__(BLOCK_THREADS, 2) k_step_block(const StepArgs<
         }
         if constexpr (!LAST) __syncthreads();
     });
+}
+
+// Whether tiles step the lattice faster than one launch per step does (sms: the device's SMs).  us a step, one by one /
+// in tiles, Newtonian Yu and Smagorinsky Chai (N, S) unless named:
+//  - Tiles that are all resident at once always do: a step launch takes 2.4 us or more (periodic 257x300 N 2.7 / 1.9, S
+//    3.0 / 2.7; 3x6000 N 3.3 / 2.6; 6000x1 N 2.6 / 2.3 but S 2.5 / 2.9).
+//  - Otherwise not where they compute a third more positions than the one-step grid: 20000x5 periodic S 3.1 / 6.3,
+//    20000x41 cavity S 8.5 / 10.3, 20000x45 8.9 / 8.9, 65x20000 cavity N 21 / 20.
+//  - Between walls they do at any size (700^2 N 6.7 / 5.5, S 7.9 / 7.4; 1000^2 10.3 / 9.3, 12.2 / 12.3; 4096^2 177 / 129,
+//    182 / 164), except forced Smagorinsky flow above two waves of blocks (512^2 6.0 / 5.2, 1000^2 13.5 / 14.5,
+//    4096^2 193 / 208).
+//  - Periodic (or walled one way): the one-step grid has no branches at walls, and while both buffers stay in L2 it is the
+//    faster above two waves: 600^2 N 4.5 / 3.9, S 5.3 / 5.0; 700^2 5.8 / 5.5, 6.5 / 7.1; 1000^2 9.3 / 9.5, 10.3 / 12.1.  From
+//    HBM tiles pay again for the fixed rates and the deviatoric closure (2048^2 N 45.7 / 36.2, deviatoric Yu 45.9 /
+//    39.9), not for the others (S 48.0 / 49.9).  L2 holds 129 MB; at 104 MB (1200^2) N 14.5 / 13.0.
+//  - The power law is bound by its sweeps, which margins repeat: up to 2^19 nodes (cavity n = 0.5 Yu: 512^2 6.5 / 5.5,
+//    1000^2 14.4 / 15.8, 4096^2 200 / 218), periodic up to one and a half waves (512^2 n = 0.6 5.7 / 5.4, 600^2 6.6 / 6.9);
+//    with n = 1, which takes no sweeps, also between walls without a force from HBM (4096^2 Yu 179 / 161, Chai 181 /
+//    173; but 1000^2 11.5 / 12.0, forced 4096^2 193 / 196).
+inline bool block_pays(const StepArgs<float>& a, int closure, int force, int sms) {
+    const long long N = (long long)a.nx * a.ny, tiles = (a.nx + BW - 1LL) / BW * ((a.ny + 19LL) / 20);
+    const bool walls = (a.wall_mask & 3) && (a.wall_mask & 12);
+    const bool from_hbm = 2LL * 9 * (int)sizeof(float) * a.stride > (96LL << 20), power_law = closure == CL_POWERLAW;
+    if (power_law && N > (1LL << 19) && !(a.pl_nm1 == 0.0f && walls && !force && from_hbm)) return false;
+    if (tiles <= 2LL * sms) return true;
+    dim3 g, b;
+    lattice_grid(a.nx, a.ny, 1, &g, &b);
+    if (10 * tiles * BW * 20 > 13LL * g.x * b.x * g.y * b.y) return false;
+    if (walls && !(closure == CL_SMAG && force)) return true;
+    if (tiles <= (power_law ? 3LL : 4LL) * sms) return true;
+    return from_hbm && (closure == CL_NEWTON || closure == CL_SMAG_DEV);
 }
 
 template <int C, int F, bool FO, int BH>

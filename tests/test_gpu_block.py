@@ -50,3 +50,38 @@ def test_lagged_closure_and_large_power_law_lattices_step_one_by_one():
         c = Case(9, dims, precision="fp32", closure=closure, tau=0.6, pl=(0.7, 0.01))
         c.lat.init(c.drho, c.u, c.g).step(8)
         assert c.lat.stats() == (8, 8)
+
+
+WALLED = dict(bc=["wall"] * 4)
+ROUTES = [  # dims, closure, what else, whether tiles are taken: they are where they step faster (step_block.cuh)
+    ((256, 256), "newton", {}, True),
+    ((600, 600), "newton", {}, True),
+    ((700, 700), "newton", {}, False),
+    ((1000, 1000), "newton", {}, False),
+    ((1000, 1000), "newton", WALLED, True),
+    ((1000, 1000), "smag", WALLED, True),
+    ((1000, 1000), "smag", dict(force=[1e-6, 0], **WALLED), False),
+    ((1000, 1000), "smag_dev", dict(force=[1e-6, 0], **WALLED), True),
+    ((1500, 1400), "newton", dict(force=[1e-6, 0]), True),
+    ((1500, 1400), "smag", {}, False),
+    ((1500, 1400), "smag_dev", {}, True),
+    ((1, 20000), "newton", {}, False),
+    ((20000, 1), "newton", {}, False),
+    ((20000, 5), "smag", WALLED, False),
+    ((28, 20000), "newton", WALLED, True),
+    ((3, 6000), "newton", {}, True),
+    ((512, 512), "powerlaw", dict(pl=(0.6, 0.01)), True),
+    ((600, 600), "powerlaw", dict(pl=(0.6, 0.01)), False),
+    ((700, 700), "powerlaw", dict(pl=(0.6, 0.01), **WALLED), True),
+    ((1000, 1000), "powerlaw", dict(pl=(1.0, 0.01), **WALLED), False),
+    ((1500, 1400), "powerlaw", dict(pl=(1.0, 0.01), **WALLED), True),
+    ((1500, 1400), "powerlaw", dict(pl=(1.0, 0.01), force=[1e-6, 0], **WALLED), False),
+    ((1500, 1400), "powerlaw", dict(pl=(1.0, 0.01)), False),
+]
+
+
+@pytest.mark.parametrize("dims,closure,extra,tiles", ROUTES)
+def test_tiles_are_taken_where_they_step_faster(dims, closure, extra, tiles):
+    c = Case(9, dims + (1,), precision="fp32", closure=closure, tau=0.6, **extra)
+    c.lat.init(c.drho, c.u).step(8)
+    assert c.lat.stats() == (8, 2 if tiles else 8)
