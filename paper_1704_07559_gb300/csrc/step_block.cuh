@@ -125,21 +125,22 @@ __global__ void __launch_bounds__(BLOCK_THREADS, 2) k_step_block(const StepArgs<
 //    faster above two waves: 600^2 N 4.5 / 3.9, S 5.3 / 5.0; 700^2 5.8 / 5.5, 6.5 / 7.1; 1000^2 9.3 / 9.5, 10.3 / 12.1.  From
 //    HBM tiles pay again for the fixed rates and the deviatoric closure (2048^2 N 45.7 / 36.2, deviatoric Yu 45.9 /
 //    39.9), not for the others (S 48.0 / 49.9).  L2 holds 129 MB; at 104 MB (1200^2) N 14.5 / 13.0.
-//  - The power law is bound by its sweeps, which margins repeat: up to 2^19 nodes (cavity n = 0.5 Yu: 512^2 6.5 / 5.5,
-//    1000^2 14.4 / 15.8, 4096^2 200 / 218), periodic up to one and a half waves (512^2 n = 0.6 5.7 / 5.4, 600^2 6.6 / 6.9);
-//    with n = 1, which takes no sweeps, also between walls without a force from HBM (4096^2 Yu 179 / 161, Chai 181 /
-//    173; but 1000^2 11.5 / 12.0, forced 4096^2 193 / 196).
+//  - The power law is bound by its sweeps, which margins repeat: up to 2^19 nodes (cavity n = 0.5 Yu: 512^2 6.3 / 5.7,
+//    1000^2 14.4 / 15.8, 4096^2 200 / 218), periodic up to one and a half waves (512^2 n = 0.6 5.7 / 5.4, 600^2 6.6 / 6.9).
+//    With n = 1 it takes none (cavity Yu 1000^2 11.0 / 11.2, 4096^2 179 / 161, forced 190 / 180; periodic Chai 600^2
+//    5.1 / 4.8, 1000^2 10.3 / 12.1, 4096^2 176 / 178).
 inline bool block_pays(const StepArgs<float>& a, int closure, int force, int sms) {
     const long long N = (long long)a.nx * a.ny, tiles = (a.nx + BW - 1LL) / BW * ((a.ny + 19LL) / 20);
     const bool walls = (a.wall_mask & 3) && (a.wall_mask & 12);
-    const bool from_hbm = 2LL * 9 * (int)sizeof(float) * a.stride > (96LL << 20), power_law = closure == CL_POWERLAW;
-    if (power_law && N > (1LL << 19) && !(a.pl_nm1 == 0.0f && walls && !force && from_hbm)) return false;
+    const bool from_hbm = 2LL * 9 * (int)sizeof(float) * a.stride > (96LL << 20);
+    const bool sweeps = closure == CL_POWERLAW && a.pl_nm1 != 0.0f;
+    if (sweeps && N > (1LL << 19)) return false;
     if (tiles <= 2LL * sms) return true;
     dim3 g, b;
     lattice_grid(a.nx, a.ny, 1, &g, &b);
     if (10 * tiles * BW * 20 > 13LL * g.x * b.x * g.y * b.y) return false;
     if (walls && !(closure == CL_SMAG && force)) return true;
-    if (tiles <= (power_law ? 3LL : 4LL) * sms) return true;
+    if (tiles <= (sweeps ? 3LL : 4LL) * sms) return true;
     return from_hbm && (closure == CL_NEWTON || closure == CL_SMAG_DEV);
 }
 

@@ -73,9 +73,8 @@ ROUTES = [  # dims, closure, what else, whether tiles are taken: they are where 
     ((512, 512), "powerlaw", dict(pl=(0.6, 0.01)), True),
     ((600, 600), "powerlaw", dict(pl=(0.6, 0.01)), False),
     ((700, 700), "powerlaw", dict(pl=(0.6, 0.01), **WALLED), True),
-    ((1000, 1000), "powerlaw", dict(pl=(1.0, 0.01), **WALLED), False),
-    ((1500, 1400), "powerlaw", dict(pl=(1.0, 0.01), **WALLED), True),
-    ((1500, 1400), "powerlaw", dict(pl=(1.0, 0.01), force=[1e-6, 0], **WALLED), False),
+    ((1000, 1000), "powerlaw", dict(pl=(1.0, 0.01), **WALLED), True),
+    ((1500, 1400), "powerlaw", dict(pl=(1.0, 0.01), force=[1e-6, 0], **WALLED), True),
     ((1500, 1400), "powerlaw", dict(pl=(1.0, 0.01)), False),
 ]
 
