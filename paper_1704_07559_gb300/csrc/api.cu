@@ -281,15 +281,16 @@ cudaError_t step_by_step(lbm_ctx* c, int n, long long* launches) {
     set_buffers(c, &a[0], c->buf[0], c->buf[1]);
     set_buffers(c, &a[1], c->buf[1], c->buf[0]);
     const int force = has_force(c) ? 1 : 0;
-    bool blocks = false;  // BLOCK_STEPS to a launch (step_block.cuh): FP32 D2Q9 on the automatic schedule
-    if constexpr (std::is_same<R, float>::value)
-        blocks = c->q == 9 && c->schedule == LBM_SCHEDULE_AUTO && n >= lbm::BLOCK_STEPS &&
-                 lbm::block_d2q9_f32_pays(a[0], c->p.closure, force);
+    int rows = 0;  // of tiles that take BLOCK_STEPS to a launch (step_block.cuh): FP32 D2Q9 on the automatic schedule
+    if constexpr (std::is_same<R, float>::value) {
+        if (c->q == 9 && c->schedule == LBM_SCHEDULE_AUTO && n >= lbm::BLOCK_STEPS)
+            rows = lbm::block_d2q9_f32_rows(a[0], c->p.closure, c->p.formula, force);
+    }
     for (int it = 0; it < n;) {
-        const int k = blocks && n - it >= lbm::BLOCK_STEPS ? lbm::BLOCK_STEPS : 1;
+        const int k = rows && n - it >= lbm::BLOCK_STEPS ? lbm::BLOCK_STEPS : 1;
         cudaError_t e = cudaErrorInvalidValue;
         if constexpr (std::is_same<R, float>::value) {
-            if (k > 1) e = lbm::block_d2q9_f32(a[c->cur], c->p.closure, c->p.formula, force, c->stream);
+            if (k > 1) e = lbm::block_d2q9_f32(a[c->cur], rows, c->p.closure, c->p.formula, force, c->stream);
         }
         if (k == 1) e = launch_step(c, a[c->cur], force);
         if (e != cudaSuccess) return e;

@@ -3,24 +3,30 @@
 
 namespace lbm {
 
-// Not for the lagged closure, whose stored tau the margins would each advance
-bool block_d2q9_f32_pays(const StepArgs<float>& a, int closure, int force) {
-    int dev = 0, sms = 0;
-    if (closure == CL_SMAG_LAGGED || cudaGetDevice(&dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
-        return false;
-    return block_pays(a, closure, force, sms);
+static cudaError_t dispatch(const StepArgs<float>& a, int rows, int closure, int formula, int force, bool prepare,
+                            cudaStream_t s) {
+    switch (closure) {
+        case CL_NEWTON: return launch_block_c<CL_NEWTON>(a, rows, formula, force, prepare, s);
+        case CL_SMAG: return launch_block_c<CL_SMAG>(a, rows, formula, force, prepare, s);
+        case CL_POWERLAW: return launch_block_c<CL_POWERLAW>(a, rows, formula, force, prepare, s);
+        case CL_SMAG_DEV: return launch_block_c<CL_SMAG_DEV>(a, rows, formula, force, prepare, s);
+        default: return cudaErrorNotSupported;  // the lagged closure's stored tau the margins would each advance
+    }
 }
 
-// BLOCK_STEPS steps from a's source to its destination
-cudaError_t block_d2q9_f32(const StepArgs<float>& a, int closure, int formula, int force, cudaStream_t s) {
-    switch (closure) {
-        case CL_NEWTON: return launch_block_c<CL_NEWTON>(a, formula, force, s);
-        case CL_SMAG: return launch_block_c<CL_SMAG>(a, formula, force, s);
-        case CL_POWERLAW: return launch_block_c<CL_POWERLAW>(a, formula, force, s);
-        case CL_SMAG_DEV: return launch_block_c<CL_SMAG_DEV>(a, formula, force, s);
-        default: return cudaErrorNotSupported;
-    }
+int block_d2q9_f32_rows(const StepArgs<float>& a, int closure, int formula, int force) {
+    int dev = 0, sms = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+        return 0;
+    if (!block_pays(a, closure, force, sms)) return 0;
+    const long long tiles = (a.nx + BW - 1LL) / BW * ((a.ny + 19LL) / 20);
+    const int rows = tiles >= sms ? 20 : 16;
+    return dispatch(a, rows, closure, formula, force, true, nullptr) == cudaSuccess ? rows : 0;
+}
+
+cudaError_t block_d2q9_f32(const StepArgs<float>& a, int rows, int closure, int formula, int force, cudaStream_t s) {
+    return dispatch(a, rows, closure, formula, force, false, s);
 }
 
 }  // namespace lbm

@@ -83,7 +83,8 @@ struct StreamCtl {
     RowWalk walk;    // how a block's threads walk a unit's rows (filled by the launcher)
 };
 
-constexpr int SUM_BLOCKS = 608;  // 4 blocks per SM on 152 SMs; partial rows in scratch
+constexpr int SUM_PER_SM = 4;               // blocks of the sums that an SM holds together
+constexpr int SUM_BLOCKS = 152 * SUM_PER_SM;  // partial rows in scratch: every block resident on a GB300's 152 SMs
 
 // The populations crossing the z faces of a slab (k_halo.cu): population up[k] (c_z = +1) of the
 // top own plane z_hi and population dn[k] (c_z = -1) of the bottom own plane z_lo, each plane
@@ -123,10 +124,11 @@ LBM_DECLARE_STREAM_ENTRY(d3q15_f16, float)
 LBM_DECLARE_STREAM_ENTRY(d3q15_bf16, float)
 LBM_DECLARE_STREAM_ENTRY(d2q9_f32, float)
 #undef LBM_DECLARE_STREAM_ENTRY
-// BLOCK_STEPS steps per launch in shared-memory tiles (step_block.cuh), and whether that is the faster form
+// BLOCK_STEPS steps per launch in shared-memory tiles (step_block.cuh), from a's source to its destination.  The rows of
+// a tile, with the current context made ready for them; 0 where one launch per step is the faster form
 constexpr int BLOCK_STEPS = 4;
-bool block_d2q9_f32_pays(const StepArgs<float>& a, int closure, int force);
-cudaError_t block_d2q9_f32(const StepArgs<float>& a, int closure, int formula, int force, cudaStream_t s);
+int block_d2q9_f32_rows(const StepArgs<float>& a, int closure, int formula, int force);
+cudaError_t block_d2q9_f32(const StepArgs<float>& a, int rows, int closure, int formula, int force, cudaStream_t s);
 // ring launches (each step writes a buffer of its own): D3Q19 FP32, Newtonian and Smagorinsky
 cudaError_t stream_ring_d3q19_f32(const StepArgs<float>& a, const StreamCtl& c, int closure, int formula, int force,
                                   int force_stream, cudaStream_t s);

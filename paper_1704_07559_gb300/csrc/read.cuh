@@ -103,7 +103,8 @@ __device__ __forceinline__ void sum_node(const StepArgs<R>& a, const R (&f)[L::Q
 
 // FP32 is held to 64 registers, so that the grid's four blocks per SM are resident together.
 template <class L, class ST>
-__global__ void __launch_bounds__(SUM_THREADS, sizeof(typename Store<ST>::R) == 4 ? SUM_BLOCKS / 152 : 0) k_sums(const StepArgs<typename Store<ST>::R> a, double* __restrict__ partial) {
+__global__ void __launch_bounds__(SUM_THREADS, sizeof(typename Store<ST>::R) == 4 ? SUM_PER_SM : 0)
+    k_sums(const StepArgs<typename Store<ST>::R> a, double* __restrict__ partial) {
     using R = typename Store<ST>::R;
     constexpr int D = L::D;
     constexpr bool AHEAD = sizeof(R) == 4;

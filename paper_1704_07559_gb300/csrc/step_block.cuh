@@ -21,8 +21,6 @@
 // law n = 0.5, 700^2 Yu 10.9 / 9.7 / 9.5, with 52 bytes spilled).
 #pragma once
 
-#include <atomic>
-
 #include "launch.h"
 #include "step.cuh"
 
@@ -144,32 +142,27 @@ inline bool block_pays(const StepArgs<float>& a, int closure, int force, int sms
     return from_hbm && (closure == CL_NEWTON || closure == CL_SMAG_DEV);
 }
 
+// Either launches the tiles or (prepare) raises the kernel's shared-memory limit, which belongs to the current CUDA
+// context and so is set by every lbm_step call that takes tiles
 template <int C, int F, bool FO, int BH>
-cudaError_t launch_block_tile(const StepArgs<float>& a, cudaStream_t s) {
+cudaError_t launch_block_tile(const StepArgs<float>& a, bool prepare, cudaStream_t s) {
     auto* k = k_step_block<D2Q9, C, F, FO, BH>;
-    // the kernel's shared-memory limit is set once per device
-    static std::atomic<unsigned long long> ready{0};
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return e;
-    if (dev >= 64 || !((ready.load() >> dev) & 1)) {
-        e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, block_smem(BH));
-        if (e != cudaSuccess) return e;
-        if (dev < 64) ready.fetch_or(1ull << dev);
-    }
+    if (prepare) return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, block_smem(BH));
     const dim3 grid((a.nx + BW - 1) / BW, (a.ny + BH - 1) / BH);
     return launch_pdl_smem(k, grid, dim3(BLOCK_THREADS), block_smem(BH), s, a);
 }
 template <int C, int F, bool FO>
-cudaError_t launch_block_form(const StepArgs<float>& a, cudaStream_t s) {
-    const long long tiles = (a.nx + BW - 1LL) / BW * ((a.ny + 19LL) / 20);
-    return tiles >= 152 ? launch_block_tile<C, F, FO, 20>(a, s) : launch_block_tile<C, F, FO, 16>(a, s);
+cudaError_t launch_block_form(const StepArgs<float>& a, int rows, bool prepare, cudaStream_t s) {
+    return rows == 20 ? launch_block_tile<C, F, FO, 20>(a, prepare, s) : launch_block_tile<C, F, FO, 16>(a, prepare, s);
 }
 
 template <int C>
-cudaError_t launch_block_c(const StepArgs<float>& a, int formula, int force, cudaStream_t s) {
-    if (formula == F_YU) return force ? launch_block_form<C, F_YU, true>(a, s) : launch_block_form<C, F_YU, false>(a, s);
-    return force ? launch_block_form<C, F_CHAI, true>(a, s) : launch_block_form<C, F_CHAI, false>(a, s);
+cudaError_t launch_block_c(const StepArgs<float>& a, int rows, int formula, int force, bool prepare, cudaStream_t s) {
+    if (formula == F_YU)
+        return force ? launch_block_form<C, F_YU, true>(a, rows, prepare, s)
+                     : launch_block_form<C, F_YU, false>(a, rows, prepare, s);
+    return force ? launch_block_form<C, F_CHAI, true>(a, rows, prepare, s)
+                 : launch_block_form<C, F_CHAI, false>(a, rows, prepare, s);
 }
 
 }  // namespace lbm
