@@ -308,11 +308,11 @@ __device__ __forceinline__ void adjoint_unit(const AdjArgs<typename Store<ST>::R
     }
 }
 
-// Bound to 8 resident blocks per SM (64 registers, a few spilled values): 128^3, T = 64, every state kept, 9.83 ms
+// Smagorinsky bound to 8 resident blocks per SM (64 registers, 8 bytes spilled): 128^3, T = 64, every state kept, 9.83 ms
 // against 9.92 at 7 (the reverse step waits on memory; more warps hide it).  Bound by HBM: 264 B a node and
-// step at 86-90% of the copy bandwidth.
+// step at 86-90% of the copy bandwidth.  Newtonian to 7: at 8 it spilled 112 bytes (8.90 ms against 9.17).
 template <class ST, int CLOSURE>
-__global__ void __launch_bounds__(128, 8) k_adjoint_stream(const AdjArgs<typename Store<ST>::R> a0,
+__global__ void __launch_bounds__(128, CLOSURE == CL_NEWTON ? 7 : 8) k_adjoint_stream(const AdjArgs<typename Store<ST>::R> a0,
                                                         const AdjArgs<typename Store<ST>::R> a1, const StreamCtl c) {
     stream_schedule(a0.st.ny, a0.st.nz, c, [&](int k, int z, int y0, int y1) {
         const long long es = -(long long)k * c.ring;

@@ -27,12 +27,15 @@ static cudaError_t step_impl(const AdjArgs<typename Store<ST>::R>& a, int closur
 }
 
 // several adjoint steps per launch, with the forward multi-step launch's policy: lattices up to
-// 2^23 nodes with enough units that no block waits, unless forced
+// 2^23 nodes with enough units that no block waits, unless forced.  The Newtonian step is short enough that one launch
+// per step is the faster at every size (whole calls, every state kept, in one launch / one by one, ms: 112^3 T = 32 3.35 /
+// 3.22, 128^3 T = 64 8.81 / 8.67, 160^3 T = 32 9.56 / 9.16, 256x128x128 T = 16 5.08 / 4.78); the Smagorinsky one's 120^3
+// T = 32 4.17 / 4.21, 128^3 9.41 / 9.51, 160^3 9.93 / 9.81.
 template <int CLOSURE>
 static cudaError_t stream_impl(const AdjArgs<float>& a0, const AdjArgs<float>& a1, const StreamCtl& c,
                                bool force_stream, cudaStream_t s) {
     const long long N = (long long)a0.st.nx * a0.st.ny * a0.st.nz;
-    if (!force_stream && N > (1LL << 23)) return cudaErrorNotSupported;
+    if (!force_stream && (CLOSURE == CL_NEWTON || N > (1LL << 23))) return cudaErrorNotSupported;
     static const int resident = resident_blocks(k_adjoint_stream<float, CLOSURE>);
     StreamCtl u;
     if (!pick_units(c, a0.st.ny, a0.st.nz, resident, &u) && !force_stream) return cudaErrorNotSupported;

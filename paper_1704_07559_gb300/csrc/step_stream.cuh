@@ -198,10 +198,11 @@ __global__ void __launch_bounds__(128, PAIR_MIN_BLOCKS) k_step_stream_pair(const
     stream_steps<L, ST, CLOSURE, FORMULA, FORCE, true>(a0, a1, c);
 }
 
-// Ring launch (see stream_steps), one node per thread; 9 resident blocks for the Yu route (the
-// adjoint's recompute: its whole call 0.7% shorter than with 8).
+// Ring launch (see stream_steps), one node per thread.  Yu route: 9 resident blocks with the Smagorinsky closure (the
+// adjoint's recompute: its whole call 0.7% shorter than with 8), 8 with fixed rates, where 9 spilled 44 to 96 bytes
+// (128^3, T = 64, segments of 8: 11.48 ms against 11.35 at 8).
 template <class L, class ST, int CLOSURE, int FORMULA, bool FORCE>
-__global__ void __launch_bounds__(128, FORMULA == F_YU ? 9 : 7)
+__global__ void __launch_bounds__(128, FORMULA == F_YU ? (CLOSURE == CL_NEWTON ? 8 : 9) : 7)
     k_step_stream_ring(const StepArgs<typename Store<ST>::R> a, const StreamCtl c) {
     stream_schedule(a.ny, a.nz, c, [&](int k, int z, int y0, int y1) {
         const long long sh = k * c.ring;
