@@ -375,11 +375,14 @@ cudaError_t run_macro(lbm_ctx* c, void* drho, void* u) {
 // *launches counts the step kernels launched.
 constexpr int STREAM_CHUNK = 4096;
 
+int stream_chunk(const lbm_ctx* c) {
+    return (int)std::min<long long>(STREAM_CHUNK, 0x7fffffffLL / ((long long)c->nz * c->stream_tiles));
+}
+
 cudaError_t advance(lbm_ctx* c, int n, long long* launches) {
     int it = 0;
     if (n >= 2) {
-        const long long units = (long long)c->nz * c->stream_tiles;
-        const int chunk = (int)std::min<long long>(std::min(n, STREAM_CHUNK), 0x7fffffffLL / units);
+        const int chunk = std::min(n, stream_chunk(c));
         while (n - it >= 2 && chunk >= 2) {
             const int k = std::min(chunk, n - it);
             cudaError_t e = run_stream(c, k);
@@ -563,17 +566,22 @@ cudaError_t adjoint_run(lbm_ctx* c, int T, int seg, bool keep_all, char* work, c
     const long long ring = (long long)(L.state / c->elem_bytes);  // elements between segment states
     const int forced = c->schedule == LBM_SCHEDULE_STREAM ? 1 : 0;
     // n steps from the state `first`, each written to the next of the equally spaced state buffers after it:
-    // in one ring launch (FP32, where the schedule allows) or step by step
+    // in ring launches of at most stream_chunk steps (FP32, where the schedule allows) or step by step
     auto run_along = [&](char* first, int n) -> cudaError_t {
         cudaError_t err;
         if constexpr (!F64) {
-            if (n >= 2 && c->schedule != LBM_SCHEDULE_PER_STEP) {
+            const int chunk = c->schedule == LBM_SCHEDULE_PER_STEP ? 0 : stream_chunk(c);
+            while (n >= 2 && chunk >= 2) {
                 lbm::StepArgs<float> ra;
                 fill_args(c, &ra);
                 set_buffers(c, &ra, first, first + L.state);
-                const lbm::StreamCtl ctl = {c->sync, n, c->stream_rows, c->stream_tiles, 0, ring};
+                const int k = std::min(n, chunk);
+                const lbm::StreamCtl ctl = {c->sync, k, c->stream_rows, c->stream_tiles, 0, ring};
                 err = lbm::stream_ring_d3q19_f32(ra, ctl, c->p.closure, c->p.formula, has_force(c) ? 1 : 0, forced, s);
-                if (err != cudaErrorNotSupported) return err;
+                if (err == cudaErrorNotSupported) break;
+                if (err != cudaSuccess) return err;
+                first += k * L.state;
+                n -= k;
             }
         }
         for (int i = 0; i < n; ++i) {
@@ -612,11 +620,6 @@ cudaError_t adjoint_run(lbm_ctx* c, int T, int seg, bool keep_all, char* work, c
         for (int k0 = 0; k0 < T && !keep_all; k0 += seg) {
             const int k1 = (k0 + seg < T) ? k0 + seg : T;
             const bool to_cp = k1 < T;
-            if (to_cp && k1 - k0 == 1) {  // one-step segments: checkpoint to checkpoint
-                e = run_step(c, cp(k0 / seg), cp(k1 / seg));
-                if (e != cudaSuccess) return e;
-                continue;
-            }
             if (!to_cp && k1 - k0 >= 2) {  // the last segment
                 e = fill_segment(k0 / seg, k1 - k0);
                 if (e != cudaSuccess) return e;

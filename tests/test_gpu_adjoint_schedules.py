@@ -1,5 +1,7 @@
 """lbm_adjoint by its ways of launching and of keeping states: the same steps on the same states, so the functional, the
 gradient and the final state are equal bit for bit."""
+import ctypes
+
 import numpy as np
 import pytest
 import torch
@@ -42,3 +44,23 @@ def test_schedules_agree(dims, closure, formula):
     for schedule in ("stream", "auto"):
         assert same(run(lat, f0, 13, 4, schedule), ref)
         assert same(run(lat, f0, 13, None, schedule), ref)
+
+
+def test_every_state_of_a_long_run_kept():
+    """More steps than one multi-step launch takes (4096), through the C ABI with a workspace that holds every state."""
+    T, seg = 4200, 64
+    lat, f0 = lattice((16, 4, 3))
+    ref = run(lat, f0, T, seg, "per_step")
+    need = ctypes.c_int64()
+    lat._check(lbm.lib().lbm_adjoint_workspace(lat.ctx, T, seg, ctypes.byref(need)))
+    state = -(-19 * lat.stride * 4 // 256) * 256
+    nbytes = need.value + T * state
+    work = torch.empty(nbytes + 256, dtype=torch.uint8, device="cuda")
+    grad, loss = torch.empty_like(ref[1]), ctypes.c_double()
+    for schedule in ("stream", "per_step"):
+        lat.set_schedule(schedule)
+        lat.set_state(f0)
+        lat._check(lbm.lib().lbm_adjoint(lat.ctx, T, seg, ctypes.c_void_p(work.data_ptr() + (-work.data_ptr()) % 256), nbytes,
+                                         ctypes.c_void_p(grad.data_ptr()), ctypes.byref(loss)))
+        lat.status()
+        assert same((loss.value, grad, lat.get_state()), ref)
