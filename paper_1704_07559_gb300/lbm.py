@@ -277,11 +277,11 @@ class Lattice:
 
     def adjoint(self, T, seg=None):
         """(L, dL/dg) after T steps from the current state: L as a float, dL/dg as a float64
-        tensor (d, nz, ny, nx).  seg defaults to round(sqrt(T)); then, where T states take at most an
-        eighth of the device's memory and that much is free, all of them are kept instead of recomputing
-        each segment (the same result, T forward steps instead of about 2T).  A given seg bounds the
-        memory as lbm_adjoint_workspace states it.  The current state afterwards is the state after
-        T steps."""
+        tensor (d, nz, ny, nx).  seg defaults to round(sqrt(T)); then, where T states take at most a 64th
+        of the device's memory, or at most an eighth of it and a quarter of what is free, all of them
+        are kept instead of recomputing each segment (the same result, T forward steps instead of about
+        2T).  A given seg bounds the memory as lbm_adjoint_workspace states it, to about 2 sqrt(T) states
+        for seg = round(sqrt(T)).  The current state afterwards is the state after T steps."""
         L = lib()
         T, given = int(T), seg
         seg = int(seg or max(1, round(T ** 0.5)))
@@ -291,7 +291,10 @@ class Lattice:
         if not given and 1 < T <= 1024:
             every = ctypes.c_int64()
             self._check(L.lbm_adjoint_workspace(self.ctx, T, T, ctypes.byref(every)))
-            if every.value <= torch.cuda.get_device_properties(self.device).total_memory // 8:
+            total = torch.cuda.get_device_properties(self.device).total_memory
+            # asking what is free takes 10 us, a fifteenth of a small gradient
+            if every.value <= total // 64 or (every.value <= total // 8 and
+                                              every.value <= torch.cuda.mem_get_info(self.device)[0] // 4):
                 try:
                     work = torch.empty(every.value + 256, dtype=torch.uint8, device=self.device)
                     nbytes = every

@@ -46,21 +46,60 @@ def test_schedules_agree(dims, closure, formula):
         assert same(run(lat, f0, 13, None, schedule), ref)
 
 
-def test_every_state_of_a_long_run_kept():
-    """More steps than one multi-step launch takes (4096), through the C ABI with a workspace that holds every state."""
-    T, seg = 4200, 64
-    lat, f0 = lattice((16, 4, 3))
-    ref = run(lat, f0, T, seg, "per_step")
+def kept(lat, f0, T, seg, schedule):
+    """The call with a workspace that holds every state, through the C ABI."""
     need = ctypes.c_int64()
     lat._check(lbm.lib().lbm_adjoint_workspace(lat.ctx, T, seg, ctypes.byref(need)))
-    state = -(-19 * lat.stride * 4 // 256) * 256
-    nbytes = need.value + T * state
+    size = lat.storage_dtype.itemsize
+    nbytes = need.value + T * (-(-19 * lat.stride * size // 256) * 256)
     work = torch.empty(nbytes + 256, dtype=torch.uint8, device="cuda")
-    grad, loss = torch.empty_like(ref[1]), ctypes.c_double()
+    grad = torch.empty((3,) + lat.shape, dtype=torch.float64, device="cuda")
+    loss = ctypes.c_double()
+    lat.set_schedule(schedule)
+    lat.set_state(f0)
+    lat._check(lbm.lib().lbm_adjoint(lat.ctx, T, seg, ctypes.c_void_p(work.data_ptr() + (-work.data_ptr()) % 256), nbytes,
+                                     ctypes.c_void_p(grad.data_ptr()), ctypes.byref(loss)))
+    lat.status()
+    return loss.value, grad, lat.get_state().clone()
+
+
+def test_every_state_of_a_long_run_kept():
+    """More steps than one multi-step launch takes (4096)."""
+    lat, f0 = lattice((16, 4, 3))
+    ref = run(lat, f0, 4200, 64, "per_step")
     for schedule in ("stream", "per_step"):
-        lat.set_schedule(schedule)
-        lat.set_state(f0)
-        lat._check(lbm.lib().lbm_adjoint(lat.ctx, T, seg, ctypes.c_void_p(work.data_ptr() + (-work.data_ptr()) % 256), nbytes,
-                                         ctypes.c_void_p(grad.data_ptr()), ctypes.byref(loss)))
-        lat.status()
-        assert same((loss.value, grad, lat.get_state()), ref)
+        assert same(kept(lat, f0, 4200, 64, schedule), ref)
+
+
+@pytest.mark.parametrize("precision,closure,schedule", [("fp32", "smag", "stream"), ("fp32", "newton", "per_step"),
+                                                        ("fp32", "newton", "stream"), ("fp64", "smag", "auto")])
+@pytest.mark.parametrize("T,seg", [(13, 2), (13, 4), (13, 5), (16, 4), (9, 2)])
+def test_recomputed_segments_equal_kept_states(precision, closure, schedule, T, seg):
+    """Pairs whose workspace is smaller than that of every state, so that a given seg does recompute: segments that
+    divide T, leave a remainder and leave one step."""
+    lat, f0 = lattice((96, 12, 6), precision=precision, closure=closure)
+    need, every = ctypes.c_int64(), ctypes.c_int64()
+    lat._check(lbm.lib().lbm_adjoint_workspace(lat.ctx, T, seg, ctypes.byref(need)))
+    lat._check(lbm.lib().lbm_adjoint_workspace(lat.ctx, T, T, ctypes.byref(every)))
+    assert need.value < every.value
+    assert same(run(lat, f0, T, seg, schedule), kept(lat, f0, T, seg, schedule))
+
+
+@pytest.mark.parametrize("total,free,kept", [(64, 0, True), (63, 4, True), (63, 3, False), (8, 4, True), (8, 3, False),
+                                             (7, 100, False)])
+def test_default_leaves_memory_free(monkeypatch, total, free, kept):
+    """Every state is kept where they take a 64th of the device's memory at most, or an eighth of it and a quarter of what
+    is free (both given here in multiples of what they take); the checkpoints are used otherwise."""
+    lat, f0 = lattice((16, 8, 8))
+    every = ctypes.c_int64()
+    lat._check(lbm.lib().lbm_adjoint_workspace(lat.ctx, 9, 9, ctypes.byref(every)))
+
+    class Device:
+        total_memory = total * every.value
+
+    sizes, empty = [], torch.empty
+    monkeypatch.setattr(torch, "empty", lambda *shape, **kw: sizes.append(shape[0]) or empty(*shape, **kw))
+    monkeypatch.setattr(torch.cuda, "get_device_properties", lambda d: Device)
+    monkeypatch.setattr(torch.cuda, "mem_get_info", lambda d: (free * every.value, Device.total_memory))
+    lat.adjoint(9)
+    assert (sizes[0] >= every.value) == kept
