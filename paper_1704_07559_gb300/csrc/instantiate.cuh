@@ -34,11 +34,13 @@ cudaError_t launch_form(const StepArgs<typename Store<ST>::R>& a, cudaStream_t s
         lattice_grid(a.nx, a.ny, a.nzc, &g, &b, T);
         return launch_pdl(k_step<L, ST, C, F, FO, true>, g, b, s, a, NodeMap{});
     } else {
-        // rows that nearly fill their blocks keep the plain grid only where both buffers stay in L2 (121x89x38,
-        // 62 MB: 38.6 against 36.5 GLUPS); from HBM blocks that start off a 128-byte line cost more than the
-        // two divisions (250x150x97: 39.6 against 42.5)
-        const bool in_l2 = 2LL * L::Q * a.stride * (int)sizeof(ST) <= (64LL << 20);
-        const NodeMap m = node_grid<1>(a, T, in_l2 ? 16 : 0, &g);
+        // rows that nearly fill their blocks keep the plain grid only where both buffers take at most 64 MB, half of L2
+        // (us a step, plain grid / node order: 62 MB, 121x89x38 channel, FP32 Newtonian Chai 11.0 / 11.7, FP16 Smagorinsky
+        // Yu 15.0 / 16.4; D3Q19 FP32 Smagorinsky Yu channel nx = 125 20 MB 6.9 / 7.5, 45 MB 9.9 / 10.3, 62 MB 12.4 / 12.3, but
+        // 75 MB 14.3 / 13.1, 130 MB 27.3 / 25.7, 400 MB 74 / 68): beyond, blocks that start off a 128-byte line cost
+        // more than the two divisions
+        const bool small = 2LL * L::Q * a.stride * (int)sizeof(ST) <= (64LL << 20);
+        const NodeMap m = node_grid<1>(a, T, small ? 16 : 0, &g);
         return m.nx.m == 0 ? launch_pdl(k_step<L, ST, C, F, FO, true>, g, dim3(T), s, a, m)
                            : launch_pdl(k_step<L, ST, C, F, FO, false>, g, dim3(T), s, a, m);
     }
