@@ -20,8 +20,19 @@ cudaError_t launch_form(const StepArgs<typename Store<ST>::R>& a, cudaStream_t s
     dim3 g;
     if constexpr (sizeof(ST) == 2) {
         if (a.nx % 2 == 0) {
-            const NodeMap m = node_grid<2>(a, 128, 16, &g);
-            return launch_pdl(k_step_pair_seq<L, ST, C, F, FO>, g, dim3(128), s, a, m);
+            // Between walls in y or z whole rows take the general pull, and in node order a warp across such a row and the
+            // next takes both branches: blocks of whole rows there while their idle lanes amount to less than one wave
+            // of blocks (us a step, whole rows / node order, D3Q15 FP16 Newtonian: 112x49x33 channel 10.4 / 13.3, 60x90x90
+            // 19.3 / 23.2, 200x45x69 25 / 28, but 72x90x90 25.0 / 23.1, 40x130x130 27 / 26, 24x130x130 24 / 20)
+            const int row = a.nx / 2;
+            const long long idle = ((row + 31) / 32 * 32 - row) * (long long)a.ny * a.nzc;
+            dim3 b(128);
+            NodeMap m = node_grid<2>(a, 128, 16, &g);
+            if ((a.wall_mask & 60) && idle <= (7LL << 14)) {
+                m.nx.m = 0;
+                lattice_grid(row, a.ny, a.nzc, &g, &b);
+            }
+            return launch_pdl(k_step_pair_seq<L, ST, C, F, FO>, g, b, s, a, m);
         }
     }
     // FP64 (bound by a pipe that each SM has its own share of): blocks of 64 spread a small lattice more
