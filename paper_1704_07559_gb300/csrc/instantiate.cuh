@@ -9,6 +9,18 @@
 
 namespace lbm {
 
+// Between walls in y or z whole rows take the general pull, and in node order a warp across such a row and the next
+// takes both branches.  Small lattices, whose slowest warps are their time, step there by blocks of whole rows
+// (lattice_grid) while the lanes idle at row ends are under `idle`, half a wave of blocks or, with pairs, one; FP64 never,
+// whose pipe bounds it.  us a step, whole rows / node order, channels, D3Q15: FP16 Newtonian 112x49x33 10.4 / 13.3, 60x90x90
+// 19.3 / 23.2, 200x45x69 25 / 28, but 72x90x90 25.0 / 23.1, 40x130x130 27 / 26; nx odd 63x49x33 8.1 / 9.1, 73x90x90 level; FP32
+// Smagorinsky 62x49x33 5.8 / 6.9, 120x90x90 0.92 of the time, 72x90x90 1.12.
+template <class RS>
+inline bool whole_rows(const StepArgs<RS>& a, int row, int idle, int nodes) {
+    return (a.wall_mask & 60) && (long long)a.nx * a.ny * a.nzc <= nodes &&
+           ((row + 31) / 32 * 32 - row) * (long long)a.ny * a.nzc <= idle;
+}
+
 // Step kernel selection: one node per thread (k_step), except 16-bit storage with nx even,
 // which runs two x-adjacent nodes per thread in packed FP32-pair arithmetic
 // (k_step_pair_seq, step_pair.cuh: the 16-bit step is issue-bound, and the shared pull and the
@@ -20,17 +32,11 @@ cudaError_t launch_form(const StepArgs<typename Store<ST>::R>& a, cudaStream_t s
     dim3 g;
     if constexpr (sizeof(ST) == 2) {
         if (a.nx % 2 == 0) {
-            // Between walls in y or z whole rows take the general pull, and in node order a warp across such a row and the
-            // next takes both branches: blocks of whole rows there while their idle lanes amount to less than one wave
-            // of blocks (us a step, whole rows / node order, D3Q15 FP16 Newtonian: 112x49x33 channel 10.4 / 13.3, 60x90x90
-            // 19.3 / 23.2, 200x45x69 25 / 28, but 72x90x90 25.0 / 23.1, 40x130x130 27 / 26, 24x130x130 24 / 20)
-            const int row = a.nx / 2;
-            const long long idle = ((row + 31) / 32 * 32 - row) * (long long)a.ny * a.nzc;
             dim3 b(128);
             NodeMap m = node_grid<2>(a, 128, 16, &g);
-            if ((a.wall_mask & 60) && idle <= (7LL << 14)) {
+            if (whole_rows(a, a.nx / 2, 7 << 14, 1 << 21)) {
                 m.nx.m = 0;
-                lattice_grid(row, a.ny, a.nzc, &g, &b);
+                lattice_grid(a.nx / 2, a.ny, a.nzc, &g, &b);
             }
             return launch_pdl(k_step_pair_seq<L, ST, C, F, FO>, g, b, s, a, m);
         }
@@ -51,9 +57,14 @@ cudaError_t launch_form(const StepArgs<typename Store<ST>::R>& a, cudaStream_t s
         // 75 MB 14.3 / 13.1, 130 MB 27.3 / 25.7, 400 MB 74 / 68): beyond, blocks that start off a 128-byte line cost
         // more than the two divisions
         const bool small = 2LL * L::Q * a.stride * (int)sizeof(ST) <= (64LL << 20);
-        const NodeMap m = node_grid<1>(a, T, small ? 16 : 0, &g);
-        return m.nx.m == 0 ? launch_pdl(k_step<L, ST, C, F, FO, true>, g, dim3(T), s, a, m)
-                           : launch_pdl(k_step<L, ST, C, F, FO, false>, g, dim3(T), s, a, m);
+        dim3 b(T);
+        NodeMap m = node_grid<1>(a, T, small ? 16 : 0, &g);
+        if (sizeof(ST) != 8 && whole_rows(a, a.nx, 1 << 16, 1 << 20)) {
+            m.nx.m = 0;
+            lattice_grid(a.nx, a.ny, a.nzc, &g, &b);
+        }
+        return m.nx.m == 0 ? launch_pdl(k_step<L, ST, C, F, FO, true>, g, b, s, a, m)
+                           : launch_pdl(k_step<L, ST, C, F, FO, false>, g, b, s, a, m);
     }
 }
 

@@ -39,7 +39,7 @@ static cudaError_t stream_impl(const AdjArgs<float>& a0, const AdjArgs<float>& a
     static const int resident = resident_blocks(k_adjoint_stream<float, CLOSURE>);
     StreamCtl u;
     if (!pick_units(c, a0.st.ny, a0.st.nz, resident, &u) && !force_stream) return cudaErrorNotSupported;
-    u.walk = row_walk(a0.st.nx, false);
+    u.walk = row_walk(a0.st.nx, 0);
     const long long total = (long long)a0.st.nz * u.tiles_y * u.steps;
     if (total >= (1LL << 31) || u.steps < 1) return cudaErrorInvalidValue;
     const int grid = (int)(total < resident ? total : resident);

@@ -33,17 +33,17 @@ __device__ __forceinline__ int div_fast(int n, FastDiv d) {
 #endif
 
 // A 128-thread block walking rows of `row` positions (nx nodes, or nx / 2 pairs) in node order: each of its
-// passes moves a thread 128 positions on, dq rows and dr positions.  Pairs (`fill`) walk rows that leave at
-// most a sixteenth of their last passes' threads idle as if filled up, skipping positions beyond the row: a
+// passes moves a thread 128 positions on, dq rows and dr positions.  Pairs walk rows that leave at most 1/waste of
+// themselves idle in their last passes (0: no rows) as if filled up, skipping positions beyond the row: a
 // warp across two rows takes both rows' branches (250x150x97 channel, GLUPS, in node order / row by row:
 // FP16 57.1 / 59.3, but FP32 39.7 / 36.9).
 struct RowWalk {
     FastDiv div;
     int row, dq, dr;
 };
-inline RowWalk row_walk(int row, bool fill) {
+inline RowWalk row_walk(int row, int waste) {
     const int full = (int)((row + 127LL) / 128 * 128);
-    if (fill && full - row <= row / 16) row = full;
+    if (waste && full - row <= row / waste) row = full;
     return {fast_div((unsigned)row), row, 128 / row, 128 % row};
 }
 
