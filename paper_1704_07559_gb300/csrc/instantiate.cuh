@@ -45,7 +45,16 @@ cudaError_t launch_form(const StepArgs<typename Store<ST>::R>& a, cudaStream_t s
     // evenly over the SMs (32^3: 512 blocks over 152 SMs instead of 256)
     constexpr int T = sizeof(ST) == 8 ? 64 : 128;
     if constexpr (L::D == 2) {
-        // the lightest step: the plain grid always (1000^2, 2% of the threads idle: 97.4 GLUPS against 92.1 in
+        // FP64 rows that leave more than a 16th of their blocks idle go in node order, but for lattices of a few us: idle
+        // threads are idle FP64 pipes, and of rows of 65 to 128 nodes every second block, and so every second SM, gets
+        // little (us a step, Newtonian Yu, plain grid / node order: 66x1264 cavity 29 / 18, 96x400 12.0 / 9.0, 257x300 17.1 /
+        // 14.9, but 67x67 6.0 / 6.7)
+        if constexpr (sizeof(ST) == 8) {
+            const NodeMap m = node_grid<1>(a, T, 16, &g);
+            if (m.nx.m != 0 && (long long)a.nx * a.ny > (1 << 14))
+                return launch_pdl(k_step<L, ST, C, F, FO, false>, g, dim3(T), s, a, m);
+        }
+        // FP32, the lightest step: the plain grid always (1000^2, 2% of the threads idle: 97.4 GLUPS against 92.1 in
         // node order)
         dim3 b;
         lattice_grid(a.nx, a.ny, a.nzc, &g, &b, T);

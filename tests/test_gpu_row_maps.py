@@ -30,3 +30,11 @@ def test_every_node_is_stepped_once(q, precision, nx, bc):
     got = c.lat.set_schedule("stream").step(7).status().get_state()
     bits = torch.int16 if got.element_size() == 2 else torch.int32
     assert torch.equal(got.view(bits), ref.view(bits))
+
+
+@pytest.mark.parametrize("nx", [66, 128, 131])
+@pytest.mark.parametrize("bc", [None, ["wall"] * 4])
+def test_every_node_of_a_2d_fp64_lattice_is_stepped_once(nx, bc):
+    c = Case(9, (nx, 260, 1), precision="fp64", closure="smag", formula="chai", tau=0.55, bc=bc, force=[1e-5, 0])
+    c.check_init()
+    c.check_step()
