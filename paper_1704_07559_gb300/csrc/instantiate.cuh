@@ -11,8 +11,8 @@ namespace lbm {
 
 // Between walls in y or z whole rows take the general pull, and in node order a warp across such a row and the next
 // takes both branches.  Small lattices, whose slowest warps are their time, step there by blocks of whole rows
-// (lattice_grid) while the lanes idle at row ends are under `idle`, half a wave of blocks or, with pairs, one; FP64 never,
-// whose pipe bounds it.  us a step, whole rows / node order, channels, D3Q15: FP16 Newtonian 112x49x33 10.4 / 13.3, 60x90x90
+// (lattice_grid) while the lanes idle at row ends are under `idle`, one wave of blocks or, in FP32, half of one; FP64
+// never, whose pipe bounds it.  us a step, whole rows / node order, channels, D3Q15: FP16 Newtonian 112x49x33 10.4 / 13.3, 60x90x90
 // 19.3 / 23.2, 200x45x69 25 / 28, but 72x90x90 25.0 / 23.1, 40x130x130 27 / 26; nx odd 63x49x33 8.1 / 9.1, 73x90x90 level; FP32
 // Smagorinsky 62x49x33 5.8 / 6.9, 120x90x90 0.92 of the time, 72x90x90 1.12.
 template <class RS>
@@ -68,7 +68,7 @@ cudaError_t launch_form(const StepArgs<typename Store<ST>::R>& a, cudaStream_t s
         const bool small = 2LL * L::Q * a.stride * (int)sizeof(ST) <= (64LL << 20);
         dim3 b(T);
         NodeMap m = node_grid<1>(a, T, small ? 16 : 0, &g);
-        if (sizeof(ST) != 8 && whole_rows(a, a.nx, 1 << 16, 1 << 20)) {
+        if (sizeof(ST) != 8 && whole_rows(a, a.nx, sizeof(ST) == 2 ? 7 << 14 : 1 << 16, 1 << 20)) {
             m.nx.m = 0;
             lattice_grid(a.nx, a.ny, a.nzc, &g, &b);
         }
