@@ -186,14 +186,16 @@ int lbm_init(lbm_ctx* ctx, const double* drho, const double* u, const double* gr
 int lbm_step(lbm_ctx* ctx, int n);
 
 /* How lbm_step(n >= 2) launches its steps.
- *  LBM_SCHEDULE_AUTO      several steps per launch when the storage is FP32/FP16S/BF16S, the
- *                         lattice is 3D with at most 2^22 nodes and
- *                         more units (a z plane times a band of y rows of about 1024-4096 nodes)
- *                         than the GPU holds resident blocks; one launch per step otherwise (the
- *                         default).  On larger lattices, and on D2Q9 lattices, a step boundary
- *                         costs less than the multi-step launch's synchronisation.  FP32 D2Q9
- *                         lattices (not with the lagged closure, and with the power law, n != 1, up
- *                         to 2^19 nodes) run four steps per launch in shared-memory tiles instead.
+ *  LBM_SCHEDULE_AUTO      the default: several steps per launch when the storage is FP32/FP16S/BF16S, the
+ *                         lattice is 3D with at most 2^22 nodes, in FP32 with nx a multiple of 8, and has
+ *                         a quarter more units (a z plane times a band of y rows of about 1024-4096
+ *                         nodes) than the GPU holds resident blocks, and the two planes of units beyond
+ *                         them that a unit waits for; one launch per step otherwise, since a step
+ *                         boundary then costs less than the multi-step launch's synchronisation.
+ *                         FP32 D2Q9 lattices (not with the lagged closure) run four steps per launch in
+ *                         shared-memory tiles where those are the faster form: small ones always,
+ *                         large ones between walls or with fixed rates or the deviatoric closure, the power
+ *                         law up to 2^19 nodes unless n = 1.
  *  LBM_SCHEDULE_PER_STEP  one launch per step.
  *  LBM_SCHEDULE_STREAM    several steps per launch wherever the storage allows it (not FP64),
  *                         whatever the lattice size.

@@ -730,7 +730,7 @@ namespace lbm {
 __global__ void k_sums_final(const double* __restrict__ partial, int nblocks, int width, const int* flag,
                              double* __restrict__ out) {
     // every column at once: one barrier per level of the tree instead of one per level and column
-    // (608 rows of 4: 8 to 34 us before, 7 now), the last five levels inside the first warp
+    // (608 rows of 4: 7 us against 8 to 34), the last five levels inside the first warp
     __shared__ double red[4][256];
     const int t = threadIdx.x;
     double v[4] = {0.0, 0.0, 0.0, 0.0};

@@ -8,11 +8,11 @@
 // (m_neq holds even moments only, so both velocities of a pair get the same e),
 //   E = w g0 + 4.5 w cj (cj - cF)/rho0 + e,  O = 1.5 w (2 cj - cF),  f_a = E + O,  f_b = E - O.
 //
-// What bounds it: 180 B a node with a gradient (FP32), and the arithmetic.  In FP64 the population-
-// by-population form took about 530 FP64 operations a node on the pipe that finishes 2 a clock and SM:
-// 5.9 ms for a 192^3 FP32 box with a gradient, now 0.35 ms (its bytes take 0.19 ms at the measured copy
-// bandwidth; the error against 64 bits is unchanged, 2.5e-8).  FP64 storage runs the pair form above in FP64; the other storages run it in
-// pairs of floats (dfloat.cuh: 48 bits, rounded once to FP32 at the end, as the FP64 result was), and
+// What bounds it: 180 B a node with a gradient (FP32), and the arithmetic.  In FP64 a population-
+// by-population form takes about 530 FP64 operations a node on the pipe that finishes 2 a clock and SM:
+// 5.9 ms for a 192^3 FP32 box with a gradient against 0.35 ms in this form (its bytes take 0.19 ms at the measured copy
+// bandwidth; the error against 64 bits is 2.5e-8 either way).  FP64 storage runs the pair form above in FP64; the other
+// storages run it in pairs of floats (dfloat.cuh: 48 bits, rounded once to FP32 at the end, as the FP64 result was), and
 // only nodes next to a moving wall, with a result that is not finite or with values near the smallest of FP32
 // repeat it in FP64.
 #pragma once

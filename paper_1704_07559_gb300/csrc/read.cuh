@@ -64,9 +64,9 @@ __global__ void __launch_bounds__(128) k_macro(const StepArgs<typename Store<ST>
 // with an error-free two-sum (hi, lo) pair per component, FP64 states in plain FP64; per-block
 // partials go to scratch as FP64 and one ordered pass adds them.  A thread waits for one node's
 // populations at a time, so with FP32 arithmetic it fetches its next node's before adding the first's
-// (the order of the additions is the same): 200x150x97 FP32 channel 72 -> 57 us (its bytes: 33 us), and with
+// (the order of the additions is the same): 200x150x97 FP32 channel 57 us against 72 (its bytes: 33 us), and with
 // every block resident (80 registers left the fourth of each SM to a second round) the three read-outs of a pass
-// 199 -> 178 us.
+// 178 us against 199.
 
 constexpr int SUM_THREADS = 256;
 

@@ -161,7 +161,7 @@ __device__ __forceinline__ double r_abs(double x) { return fabs(x); }
 // Closure arithmetic: in FP32 the approximate reciprocal, reciprocal square root, logarithm and power of
 // two (errors of a few ulp, far inside the FP32 tolerance of S), in FP64 the IEEE operations.  The reciprocal and the
 // square root are the instructions that take subnormals as zero, without the scaling around them (channel
-// 256x128x128, 20 steps, Smagorinsky: FP16 Yu 61.1 -> 64.1 GLUPS, Chai 51.3 -> 53.8, FP32 Chai 41.7 -> 42.1):
+// 256x128x128, 20 steps, Smagorinsky, GLUPS with the scaling / without: FP16 Yu 61.1 / 64.1, FP32 Chai 41.7 / 42.1):
 // tau lies above 1/2, and a strain under 1.1e-19, whose square is subnormal, adds less than half a last place to
 // a tau0 of 1/2 and more for any 3 Cs^2 below 2.7e11.  So is the power of two: |S|^(n-1) is never subnormal for n up
 // to 2.69, nor seen beside 1/2 beyond that unless 3K is above 2^100.  The logarithm is not: tau of the power
@@ -936,9 +936,9 @@ __device__ __forceinline__ RS power_law_start(RS qc, const StepArgs<RS>& a) {
 // power_law.h) the sweeps start from it and one that stays inside the clamps is followed by a Newton
 // step; there F has one fixed point, so the stopping rule accepts the same one.  A sweep costs 20
 // instructions and 3 special-function ones, a Newton step 8 and 1 more: from tau0 a node needs 8 to
-// 10 sweeps and a warp 12 to 18, from the guess 3 (4096^2 cavity, n = 0.5, developed flow, FP32
-// Yu / Chai 60.2 / 58.2 -> 83.0 / 78.7 GLUPS, 1024^2 FP64 0.37 -> 1.03; a cavity at rest, where two plain
-// sweeps did, 84.2 -> 83.3).
+// 10 sweeps and a warp 12 to 18, from the guess 3 (4096^2 cavity, n = 0.5, developed flow, us a step,
+// plain sweeps / from the guess: FP32 Yu 278 / 201, Chai 288 / 209, 1024^2 FP64 2.8 / 1.0 ms; at rest, where two plain
+// sweeps do, the guess costs 1%).
 template <int CLOSURE, class RS>
 __device__ __forceinline__ RS tau_fixed_point(RS qa, RS qb2, RS qc, const StepArgs<RS>& a) {
     RS tau = a.tau0;
@@ -950,7 +950,7 @@ __device__ __forceinline__ RS tau_fixed_point(RS qa, RS qb2, RS qc, const StepAr
             tau = tn;
         }
     } else {
-        if (a.pl_nm1 == RS(0)) {  // n = 1: F does not depend on tau (two sweeps less: 1025x1023 12.9 -> 11.3 us a step)
+        if (a.pl_nm1 == RS(0)) {  // n = 1: F does not depend on tau (1025x1023 11.3 us a step, by sweeps 12.9)
             RS tn = a.pl_k3 + RS(0.5);
             if (!(tn >= a.pl_tau_min)) tn = a.pl_tau_min;
             return tn > a.pl_tau_max ? a.pl_tau_max : tn;
@@ -1514,9 +1514,9 @@ __device__ __forceinline__ void step_body(const StepArgs<typename Store<ST>::R>&
 }
 
 // Which node(s) a thread takes: PER x-adjacent nodes each (nx a multiple of PER), in node order over the
-// computed planes, so that rows of any length fill the blocks: with blocks cut at the row ends the step ran
-// (GLUPS, before -> now) FP32 200x150x97 channel 35.8 -> 40.6, 97x150x97 28.6 -> 37.1, 80^3 box 37.1 -> 45.9,
-// 301x301x199 39.0 -> 45.3, FP16 200x150x97 42.8 -> 50.9, 96^3 48.1 -> 63.8.  Where rows fill whole blocks
+// computed planes, so that rows of any length fill the blocks (GLUPS, blocks cut at the row ends / node order: FP32
+// 200x150x97 channel 35.8 / 40.6, 97x150x97 28.6 / 37.1, 80^3 box 37.1 / 45.9, 301x301x199 39.0 / 45.3, FP16
+// 200x150x97 42.8 / 50.9, 96^3 48.1 / 63.8; but see whole_rows).  Where rows fill whole blocks
 // anyway (nx.m = 0) the grid gives x, y and z directly, without the two divisions; the FP32 and FP64 steps
 // are built for each map, since choosing at run time cost them up to 8% (121x89x38 channel).
 struct NodeMap {
@@ -1565,11 +1565,12 @@ inline NodeMap node_grid(const StepArgs<RS>& a, int threads, int waste, dim3* gr
 
 // One node per thread.  The bound names no minimum of resident blocks for the 16-bit and FP32 3D lattices: a
 // minimum of one changes ptxas's register allocation (more registers, fewer resident blocks).  FP64 names one
-// that leaves it more registers than it takes unasked (128 in 3D, 64 in 2D): bound by the FP64 pipe, the step
-// gains by holding values instead of forming them again (GLUPS: D3Q19 channel Yu 1.28 -> 1.43, Newtonian box Chai
-// 2.11 -> 2.32, D3Q15 channel Yu 1.54 -> 1.63, 1000^2 D2Q9 Chai 4.88 -> 5.39; a cap of 80 in 3D 1.26).  FP32 D2Q9 is
+// that leaves it more registers than it takes unasked (up to 128 in 3D, 64 in 2D): bound by the FP64 pipe, the step
+// gains by holding values instead of forming them again (us a step, unasked / bounded: D3Q19 256x128x128 channel Yu
+// 3250 at 106 registers / 2918 at 116, 128x128x64 Newtonian box Chai 495 / 451, D3Q15 256x128x64 channel Yu 1355 / 1276,
+// 1000^2 D2Q9 Newtonian Chai 205 / 186; a cap of 80 registers in 3D was the slowest).  FP32 D2Q9 is
 // held to 16 blocks (32 registers, full occupancy; the power law spills up to 12 values there): 4096^2
-// power-law cavity, developed n = 0.5 flow, Yu / Chai 83.0 / 78.7 GLUPS, at 12 blocks 79.8 / 76.8, at 10 71.3 / 68.2.
+// power-law cavity, developed n = 0.5 flow, Yu / Chai 83 / 79 GLUPS, at 12 blocks 80 / 77, at 10 71 / 68.
 template <class L, class ST>
 constexpr int step_min_blocks() {
     if (sizeof(ST) == 8) return L::Q == 9 ? 8 : 4;

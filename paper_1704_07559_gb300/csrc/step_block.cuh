@@ -90,7 +90,8 @@ __global__ void __launch_bounds__(BLOCK_THREADS, 2) k_step_block(const StepArgs<
         float* to = sm + (CV(k) & 1) * 9 * PITCH;
         for (int t = threadIdx.x; t < W * H; t += BLOCK_THREADS) {
             const int ly = t / W + CV(k), lx = t - (t / W) * W + CV(k);
-            const int x = wx ? ox + lx : wrap_pos<SW>(ox + lx, a.nx), y = wy ? oy + ly : wrap_pos<SH>(oy + ly, a.ny);
+            const int x = wx ? ox + lx : wrap_pos<SW>(ox + lx, a.nx);
+            const int y = wy ? oy + ly : wrap_pos<SH>(oy + ly, a.ny);
             bool mine = x >= 0 && x < a.nx && y >= 0 && y < a.ny;  // false only beyond a wall
             if (LAST) mine = mine && ox + lx < a.nx && oy + ly < a.ny;  // and past a ragged end
             if (!mine) continue;

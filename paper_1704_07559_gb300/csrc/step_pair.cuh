@@ -191,9 +191,9 @@ __device__ __forceinline__ void step_pair(const StepArgs<float>& a, const F2 (&f
 }
 
 // Two x-adjacent nodes per thread (16-bit storage, nx even).  Bound to 7 resident blocks per SM
-// (72 registers) for both routes: measured on a GB300 against 8 blocks (Yu: channel -4%, 512^3 box
-// +1%; Chai: channel FP16 51.3 -> 48.9 GLUPS, D3Q15 BF16 59.5 -> 57.0, 256^3 box 62.9 -> 64.9) and, for
-// the Chai route, 6 and 5 blocks (channel 45.1 and 46.5, box 60.5).
+// (72 registers) for both routes: against 8 blocks Yu's channel gains 4% and its 512^3 box loses 1%; Chai, us a step
+// at 6 / 7 / 8 blocks: D3Q19 FP16 channel 84.8 / 87.4 / 95.3, 256^3 box 267 / 274 / 286, BF16 128^3 41.2 / 38.4 / 40.8; D3Q15
+// BF16 channel 69.4 / 68.9 / 74.4, 256^3 224 / 219 / 220, 128^3 32.2 / 31.1 / 32.3.
 constexpr int PAIR_MIN_BLOCKS = 7;
 
 template <class L, class ST, int CLOSURE, int FORMULA, bool FORCE>
