@@ -59,24 +59,28 @@ def env_int(name, default):
         return default
 
 
-def captured_traffic(kernel):
-    """DRAM bytes per lattice step of `kernel` from the committed ncu capture (the capture's bytes
-    divided by the steps its launch ran), or None when the capture is of another kernel or the
-    kernel sources changed since it was taken."""
+def capture(name):
+    """profiles/<name>: counts of a committed ncu capture, or None when the kernel sources that it names
+    changed since it was taken (their SHA-256 is recorded with it)."""
     import hashlib
 
     try:
-        with open(os.path.join(ROOT, "profiles", "roofline_traffic.json")) as fh:
+        with open(os.path.join(ROOT, "profiles", name)) as fh:
             doc = json.load(fh)
         h = hashlib.sha256()
         for src in doc["sources"]:
             with open(os.path.join(ROOT, src), "rb") as fh:
                 h.update(fh.read())
-        if doc["kernel"] == kernel and h.hexdigest() == doc["sources_sha256"]:
-            return int(doc["dram_bytes_per_step"])
+        return doc if h.hexdigest() == doc["sources_sha256"] else None
     except (OSError, ValueError, KeyError):
-        pass
-    return None
+        return None
+
+
+def captured_traffic(kernel):
+    """DRAM bytes per lattice step of `kernel` (the capture's bytes divided by the steps its launch ran), or
+    None when the capture is of another kernel or of other sources."""
+    doc = capture("roofline_traffic.json")
+    return int(doc["dram_bytes_per_step"]) if doc and doc.get("kernel") == kernel else None
 
 
 def measured_peaks():
@@ -520,13 +524,9 @@ def run_slab(args):
 
 def fp64_alu_counts():
     """FP64 flops and FP64-pipe instructions per node update of the FP64 Yu-route step kernel,
-    from the committed ncu capture (profiles/fp64_alu.json), or None."""
-    try:
-        with open(os.path.join(ROOT, "profiles", "fp64_alu.json")) as fh:
-            doc = json.load(fh)
-        return float(doc["fp64_flops_per_lup"]), float(doc["fp64_instructions_per_lup"])
-    except (OSError, ValueError, KeyError):
-        return None
+    from the committed ncu capture (profiles/fp64_alu.json), or None when it is of other sources."""
+    doc = capture("fp64_alu.json")
+    return (float(doc["fp64_flops_per_lup"]), float(doc["fp64_instructions_per_lup"])) if doc else None
 
 
 def variants(args, hbm, peaks=None):
